@@ -128,6 +128,9 @@ class MtsFunction(torch.autograd.Function):
 
     @staticmethod
     def forward(ctx, C, sim: Simulator, want_B: bool = True):
+        # an output without a cotangent arrives as None in backward instead of zeros, so a
+        # gradient of the loss alone neither fills nor contracts a field-sized tensor of zeros
+        ctx.set_materialize_grads(False)
         out = sim.forward(C.detach(), want_B=want_B, want_loss=True)
         ctx.sim = sim
         ctx.ev = out["ev"]

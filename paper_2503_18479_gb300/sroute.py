@@ -94,9 +94,14 @@ class SRouteFunction(torch.autograd.Function):
 
     @staticmethod
     def forward(ctx, svar, sr: SRoute, want_B: bool):
+        # outputs without a cotangent arrive as None in backward (no field-sized zeros)
+        ctx.set_materialize_grads(False)
         out = sr.forward(svar.detach(), want_B=want_B)
         ctx.sr = sr
-        ctx.out = out
+        # what backward reads; not the outputs themselves, which would tie their memory (the
+        # field) to a reference cycle through this context until Python's collector runs
+        ctx.out = {"ev": out["ev"], "tape": out["tape"]}
+        ctx.has = (out["B"] is not None, out["loss"] is not None)
         B = out["B"] if out["B"] is not None else torch.zeros(0, dtype=sr.b_dtype, device=sr.device)
         loss = out["loss"] if out["loss"] is not None else torch.zeros(0, dtype=torch.float64, device=sr.device)
         return B, loss
@@ -104,8 +109,8 @@ class SRouteFunction(torch.autograd.Function):
     @staticmethod
     def backward(ctx, gB, gl):
         sr, out = ctx.sr, ctx.out
-        gB = gB if (out["B"] is not None and gB is not None and gB.numel()) else None
-        gl = gl if (out["loss"] is not None and gl is not None and gl.numel()) else None
+        gB = gB if (ctx.has[0] and gB is not None and gB.numel()) else None
+        gl = gl if (ctx.has[1] and gl is not None and gl.numel()) else None
         g = sr.backward(out, grad_B=gB, grad_loss=gl)
         return g, None, None
 
