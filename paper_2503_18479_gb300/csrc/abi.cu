@@ -61,6 +61,11 @@ TableLayout table_layout(int n_struct, int n_freq) {
   return t;
 }
 
+// Sides (common.cuh): two float4 and two int32 per vertex; ten floats and an int32 per loop.
+size_t sides_bytes(int n_vertices, int n_ports) {
+  return 40 * (size_t)n_vertices + 44 * (size_t)n_ports;
+}
+
 BasisLayout basis_layout(const mts_problem* pb, mts_precision prec) {
   ProblemSums ps = problem_sums(pb, prec);
   BasisLayout b;
@@ -75,6 +80,7 @@ BasisLayout basis_layout(const mts_problem* pb, mts_precision prec) {
   b.M32hi = o; o += align256(sizeof(float) * ps.sumNN);
   b.M32lo = o; o += align256(sizeof(float) * ps.sumNN);
   b.Aop = o; o += align256(2 * (size_t)ps.sumAop);
+  b.sides = o; o += align256(sides_bytes(pb->n_vertices, pb->n_ports));
   b.status = o; o += 256;
   b.total = o;
   return b;

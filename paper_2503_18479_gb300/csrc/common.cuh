@@ -16,6 +16,7 @@
 //   Aop        bf16 tensor-core operand of H (MTS_MIXED: 3 pieces, MTS_BF16: 1),
 //              per structure [piece][p_tile][k_chunk][128 rows x 64 k] in the
 //              128-byte-swizzled K-major image of shared memory (see swz128)
+//   sides      the straight sides of every loop (struct Sides), read while H and M are built
 //   status     int32 [4]
 //
 // Tape (written by mts_solve, read by mts_superpose and mts_backward):
@@ -117,7 +118,7 @@ struct ProblemSums {
 
 struct BasisLayout {
   size_t tables = 0, M64 = 0, H = 0, Hloss64 = 0, Hloss32 = 0, HlossT32 = 0, M32hi = 0, M32lo = 0, Aop = 0,
-         status = 0, total = 0;
+         sides = 0, status = 0, total = 0;
   int h_elem = 8;
 };
 
@@ -137,6 +138,8 @@ struct TapeLayout {
 struct PlanLayout {
   size_t bop_off, unit_off, lu_off, simt_off, bytes;
 };
+
+size_t sides_bytes(int n_vertices, int n_ports);
 
 ProblemSums problem_sums(const mts_problem* pb, mts_precision prec);
 TableLayout table_layout(int n_struct, int n_freq);
@@ -198,6 +201,35 @@ namespace mts {
 // r*128 bytes, its 16-byte chunk j = kk/8 stored at chunk position j ^ (r % 8).
 __host__ __device__ inline uint32_t swz128(uint32_t r, uint32_t kk) {
   return r * 128u + ((((kk >> 3) ^ (r & 7u)) & 7u) << 4) + ((kk & 7u) << 1);
+}
+
+// Straight sides of the loops (basis.cu, write_sides), indexed by the loop's first vertex plus
+// the side's number, and what belongs to the loop as a whole.
+struct LoopInfo {
+  float ctr_hi[3], ctr_lo[3];  // centre
+  float area2[3];              // twice the vector area, components z, x, y
+  float far2;                  // squared distance from which the far form holds
+};
+struct Sides {
+  float4* start;   // start relative to the loop's centre, longest segment squared
+  float4* dir;     // end minus start, length squared
+  int32_t* first;  // first vertex of the side, relative to the loop's first vertex
+  int32_t* segs;   // segments of the side
+  LoopInfo* loop;  // [n_ports]
+  int32_t* count;  // [n_ports] sides of the loop
+};
+
+inline Sides basis_sides(char* basis, const BasisLayout& bl, int n_vertices, int n_ports) {
+  char* b = basis + bl.sides;
+  const size_t n = n_vertices;
+  Sides s;
+  s.start = reinterpret_cast<float4*>(b);
+  s.dir = s.start + n;
+  s.first = reinterpret_cast<int32_t*>(s.dir + n);
+  s.segs = s.first + n;
+  s.loop = reinterpret_cast<LoopInfo*>(s.segs + n);
+  s.count = reinterpret_cast<int32_t*>(s.loop + n_ports);
+  return s;
 }
 
 __device__ inline int find_struct_i32(const int32_t* off, int n, int64_t x) {
