@@ -256,6 +256,7 @@ static SolveArgs solve_args(const mts_problem* pb, mts_precision prec, const voi
   a.loss_weight = ev->loss_weight;
   a.loss_offset = ev->loss_offset;
   a.tol = ev->refine_tol > 0.0 ? ev->refine_tol : 1e-8;
+  a.tol_f = (float)a.tol;
   a.max_refine = ev->max_refine > 0 ? ev->max_refine : 8;
   a.sumFN = ps.sumFN;
   a.sumFL = ps.sumFL;

@@ -38,6 +38,7 @@ struct SolveArgs {
   const double* loss_weight;  // [sumFL] or nullptr
   const double* loss_offset;  // complex [sumFL] or nullptr
   double tol;
+  float tol_f;  // the same in FP32
   int max_refine;
   int64_t sumFN, sumFL;
   double* I;          // tape

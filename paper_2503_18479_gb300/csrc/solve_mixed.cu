@@ -106,7 +106,7 @@ struct SmemV4 {
   __align__(16) float yim[NM];
   __align__(16) float2 xc[NM];           // unknowns by column (FP32), permutation buffer
   __align__(16) float2 Gs[NM];           // conj(G) of a chunk of loss points
-  double red[NW];
+  df red[NW];
   float redf[NW];
   unsigned ukey[2][NW];
   unsigned umax[NW];
@@ -136,21 +136,28 @@ __device__ inline float gmax(float v, SmemV4<NM>& sm, int r) {
 }
 
 template <int NM>
-__device__ inline double gsum(double v, SmemV4<NM>& sm, int r) {
-  if constexpr (NM <= 32) {
-    for (int off = NM >> 1; off > 0; off >>= 1) v += __shfl_xor_sync(0xffffffffu, v, off, NM);
-    return v;
-  } else {
-    for (int off = 16; off > 0; off >>= 1) v += __shfl_xor_sync(0xffffffffu, v, off);
+__device__ inline df gsum(df v, SmemV4<NM>& sm, int r) {
+  const int width = NM <= 32 ? NM : 32;
+  for (int off = width >> 1; off > 0; off >>= 1) {
+    const float h = __shfl_xor_sync(0xffffffffu, v.h, off, width);
+    const float l = __shfl_xor_sync(0xffffffffu, v.l, off, width);
+    df_acc(v, h, l);
+  }
+  if constexpr (NM > 32) {
     __syncthreads();
     if ((r & 31) == 0) sm.red[r >> 5] = v;
     __syncthreads();
-    double s = 0.0;
+    v = sm.red[0];
 #pragma unroll
-    for (int q = 0; q < SmemV4<NM>::NW; ++q) s += sm.red[q];
-    return s;
+    for (int q = 1; q < SmemV4<NM>::NW; ++q) df_acc(v, sm.red[q].h, sm.red[q].l);
   }
+  return v;
 }
+
+// a complex double-float value
+struct df2 {
+  df x, y;
+};
 
 __device__ __forceinline__ float2 crecip(float2 a) {
   // hardware approximate reciprocal (one instruction, <= 1 ulp): the factors are FP32 and
@@ -174,13 +181,13 @@ __device__ __forceinline__ void cms(float2& c, float2 a, float2 b) {
 __device__ __forceinline__ float point_loss_f(int mode, float2 b, const double* t, float* gx, float* gy) {
   if (mode == 0) {
     const float a = sqrtf(b.x * b.x + b.y * b.y);
-    const float r = a - (float)t[0];
+    const float r = a - df_from(t[0]).h;
     const float s = a > 0.0f ? 2.0f * r / a : 0.0f;
     *gx = s * b.x;
     *gy = s * b.y;
     return r * r;
   }
-  const float ex = b.x - (float)t[0], ey = b.y - (float)t[1];
+  const float ex = b.x - df_from(t[0]).h, ey = b.y - df_from(t[1]).h;
   *gx = 2.0f * ex;
   *gy = 2.0f * ey;
   return ex * ex + ey * ey;
@@ -271,19 +278,20 @@ solve_mixed_v4(SolveArgs a, int64_t n_sys) {
     // derived again after the LU, so that none of them stays live across it. ----
     SysInfo si = sys_info(a, sys);
     const int N = (in_range && si.N <= NM) ? si.N : 0;
-    const double w = si.w;
-    const float w32 = (float)w;
+    const df wd = df_from(si.w);
+    const float w32 = wd.h;
     const bool real_row = r < N;
     const float* __restrict__ Mh = a.M32hi + a.t.nn_off[si.s];
     const float* __restrict__ Ml = a.M32lo + a.t.nn_off[si.s];
-    // The diagonal entry needs FP64 (w (M_rr hi + lo) - 1/(w C_r), then rounded): it is
-    // computed once per thread here, not inside the unrolled column loop, where each
-    // column's branch would run its FP64 instructions for the one lane with c == r.
+    // The diagonal entry cancels near resonance (w (M_rr hi + lo) - 1/(w C_r), then rounded):
+    // double-float, once per thread here and not inside the unrolled column loop.
     float dre = 1.0f, dimv = 0.0f;
     if (real_row) {
-      const double Cr = a.C[si.b * a.n_ports + si.k0 + r];
-      dre = (float)a.R[si.k0 + r];
-      dimv = (float)(w * ((double)__ldg(Mh + r * N + r) + (double)__ldg(Ml + r * N + r)) - 1.0 / (w * Cr));
+      const df y = df_recip_product(si.w, a.C[si.b * a.n_ports + si.k0 + r]);
+      dre = df_from(a.R[si.k0 + r]).h;
+      df d = df_mul(wd, {__ldg(Mh + r * N + r), __ldg(Ml + r * N + r)});
+      df_acc(d, -y.h, -y.l);
+      dimv = d.h + d.l;
     }
 #pragma unroll
     for (int b = 0; b < NB; ++b)
@@ -555,12 +563,15 @@ solve_mixed_v4(SolveArgs a, int64_t n_sys) {
   const bool valid = in_range && si.N <= NM;  // larger systems: solve_large.cu
   if (!valid) si.N = 0;
   const int N = si.N;
-  const double w = si.w;
-  const float w32 = (float)w;
+  const df wd = df_from(si.w);
+  const float w32 = wd.h;
   const bool real_row = r < N;
   const bool bwd = a.rhs_in != nullptr;
-  cd Dr = {0.0, 0.0};
-  if (real_row) Dr = {a.R[si.k0 + r], -1.0 / (w * a.C[si.b * a.n_ports + si.k0 + r])};
+  df Rd = {0.0f, 0.0f}, yd = {0.0f, 0.0f};  // R_r and 1/(w C_r)
+  if (real_row) {
+    Rd = df_from(a.R[si.k0 + r]);
+    yd = df_recip_product(si.w, a.C[si.b * a.n_ports + si.k0 + r]);
+  }
   const int64_t mo = a.t.nn_off[si.s];
   const float* __restrict__ Mh = a.M32hi + mo;
   const float* __restrict__ Ml = a.M32lo + mo;
@@ -631,11 +642,11 @@ solve_mixed_v4(SolveArgs a, int64_t n_sys) {
     return sm.xc[r];
   };
 
-  // accurate residual of row r with the FP32 iterate in xc: rhs_r - sum_j A_rj x_j, the
-  // sum over M_rj x_j in double-float (M = hi + lo exactly, x exact in FP32)
-  auto residual = [&](cd rhs) -> cd {
+  // accurate residual of row r with the FP32 iterate in xc: rhs_r - sum_j A_rj x_j in
+  // double-float (M = hi + lo exactly, x exact in FP32)
+  auto residual = [&](df2 rhs) -> df2 {
     const float2 xr = sm.xc[r];
-    if (!real_row) return {rhs.x - (double)xr.x, rhs.y - (double)xr.y};
+    if (!real_row) return {{rhs.x.h - xr.x, 0.0f}, {rhs.y.h - xr.y, 0.0f}};
     u64 S[2] = {0ull, 0ull}, Lo[2] = {0ull, 0ull};  // (re, im) high and low parts, 2 chains
     const u64 neg1 = pk(-1.0f, -1.0f);
     const u64* xv = reinterpret_cast<const u64*>(sm.xc);
@@ -659,16 +670,25 @@ solve_mixed_v4(SolveArgs a, int64_t n_sys) {
       }
     }
     const float2 s0 = up(S[0]), s1 = up(S[1]), l0 = up(Lo[0]), l1 = up(Lo[1]);
-    const double Sr = ((double)s0.x + (double)l0.x) + ((double)s1.x + (double)l1.x);
-    const double Si = ((double)s0.y + (double)l0.y) + ((double)s1.y + (double)l1.y);
-    const double ax = Dr.x * (double)xr.x - Dr.y * (double)xr.y;
-    const double ay = Dr.x * (double)xr.y + Dr.y * (double)xr.x;
-    return {rhs.x - ax + w * Si, rhs.y - ay - w * Sr};
+    df Sr = {s0.x, l0.x + l1.x}, Si = {s0.y, l0.y + l1.y};
+    df_acc(Sr, s1.x, 0.0f);
+    df_acc(Si, s1.y, 0.0f);
+    // re: rhs - R x.re + w Si - x.im / (w C);  im: rhs - R x.im - w Sr + x.re / (w C)
+    const df ws = df_mul(wd, Si), wr = df_mul(wd, Sr);
+    const df rx = df_mulf(Rd, xr.x), ry = df_mulf(Rd, xr.y);
+    const df yx = df_mulf(yd, xr.x), yy = df_mulf(yd, xr.y);
+    df_acc(rhs.x, ws.h, ws.l);
+    df_acc(rhs.x, -yy.h, -yy.l);
+    df_acc(rhs.x, -rx.h, -rx.l);
+    df_acc(rhs.y, -wr.h, -wr.l);
+    df_acc(rhs.y, yx.h, yx.l);
+    df_acc(rhs.y, -ry.h, -ry.l);
+    return rhs;
   };
 
   // r -= A d for the correction d in xc (FP32)
-  auto residual_update = [&](cd res, float2 dr) -> cd {
-    if (!real_row) return {res.x - dr.x, res.y - dr.y};
+  auto residual_update = [&](df2 res, float2 dr) -> df2 {
+    if (!real_row) return {{res.x.h - dr.x, 0.0f}, {res.y.h - dr.y, 0.0f}};
     u64 S0 = 0ull, S1 = 0ull;
     const u64* xv = reinterpret_cast<const u64*>(sm.xc);
     int j = 0;
@@ -682,13 +702,14 @@ solve_mixed_v4(SolveArgs a, int64_t n_sys) {
       S0 = ffma2(pk(m0, m0), xv[j], S0);
     }
     const float2 s = make_float2(up(S0).x + up(S1).x, up(S0).y + up(S1).y);
-    const float dx = (float)Dr.x, dy = (float)Dr.y;
-    const float adx = dx * dr.x - dy * dr.y - w32 * s.y;
-    const float ady = dx * dr.y + dy * dr.x + w32 * s.x;
-    return {res.x - (double)adx, res.y - (double)ady};
+    const float adx = Rd.h * dr.x + yd.h * dr.y - w32 * s.y;
+    const float ady = Rd.h * dr.y - yd.h * dr.x + w32 * s.x;
+    df_acc(res.x, -adx, 0.0f);
+    df_acc(res.y, -ady, 0.0f);
+    return res;
   };
 
-  const float tol = (float)a.tol;
+  const float tol = a.tol_f;
   const int max_it = a.max_refine;
   const int64_t ioff = si.b * a.sumFN + a.t.fn_off[si.s] + (int64_t)si.f * N;
   const bool has_obj = !bwd && a.target != nullptr;
@@ -697,35 +718,35 @@ solve_mixed_v4(SolveArgs a, int64_t n_sys) {
     const double* Ip = a.I + 2 * (ioff + r);
     x = {Ip[0], Ip[1]};
   }
-  cd u = {0.0, 0.0};
+  df2 u = {{0.0f, 0.0f}, {0.0f, 0.0f}};
   if (bwd && real_row) {
     const double* up_ = a.rhs_in + 2 * (ioff + r);
-    u = {up_[0], up_[1]};
+    u = {df_from(up_[0]), df_from(up_[1])};
   }
   bool conv_all = true;
   bool bad = false;
   const int ph0 = bwd ? 1 : 0, ph1 = (bwd || has_obj) ? 2 : 1;
 #pragma unroll 1
   for (int ph = ph0; ph < ph1; ++ph) {
-    cd rhs64 = {0.0, 0.0};
+    df2 rhs = {{0.0f, 0.0f}, {0.0f, 0.0f}};
     if (ph == 0) {
       if (real_row) {
         const double* Vp = a.V + 2 * (a.t.fn_off[si.s] + (int64_t)si.f * N + r);
-        rhs64 = {Vp[0], Vp[1]};
+        rhs = {df_from(Vp[0]), df_from(Vp[1])};
       }
     } else {
-      rhs64 = u;
+      rhs = u;
     }
-    cd xk = {0.0, 0.0};
-    cd res = rhs64;
+    df2 xd = {{0.0f, 0.0f}, {0.0f, 0.0f}};
+    df2 res = rhs;
     float dprev = 0.0f, xm0 = 0.0f;
     bool conv = max_it == 0;
 #pragma unroll 1
     for (int it = 0;; ++it) {
       float dm;
-      const float2 d = solve_perm(make_float2((float)res.x, (float)res.y), &dm);
-      xk.x += (double)d.x;
-      xk.y += (double)d.y;
+      const float2 d = solve_perm(make_float2(res.x.h + res.x.l, res.y.h + res.y.l), &dm);
+      df_acc(xd.x, d.x, 0.0f);
+      df_acc(xd.y, d.y, 0.0f);
       bool stop = it >= max_it;
       if (it == 0) {
         xm0 = dm;
@@ -740,10 +761,13 @@ solve_mixed_v4(SolveArgs a, int64_t n_sys) {
       } else {
         if (stop) break;
       }
-      res = (it == 0) ? residual(rhs64) : residual_update(res, d);
+      res = (it == 0) ? residual(rhs) : residual_update(res, d);
     }
     conv_all = conv_all && conv;
-    bad = bad || (real_row && !(isfinite(xk.x) && isfinite(xk.y)));
+    xd.x = df_norm(xd.x.h, xd.x.l);
+    xd.y = df_norm(xd.y.h, xd.y.l);
+    bad = bad || (real_row && !(isfinite(xd.x.h) && isfinite(xd.y.h)));
+    const cd xk = {df_double(xd.x), df_double(xd.y)};
     if (ph == 0) {
       x = xk;
       if (valid && real_row) {
@@ -773,8 +797,8 @@ solve_mixed_v4(SolveArgs a, int64_t n_sys) {
             const uint32_t rr = (uint32_t)(n % kTileN);
             // x = xh + xl (FP32 pair); pieces p_q = bf16(rem), rem -= p_q in FP32 (exact
             // apart from the final rounding of rem + xl, 2^-32 relative)
-            const double xv = own ? (c == 0 ? x.x : x.y) : 0.0;
-            const float xh = (float)xv, xl = (float)(xv - (double)xh);
+            const df xv = c == 0 ? xd.x : xd.y;
+            const float xh = own ? xv.h : 0.0f, xl = own ? xv.l : 0.0f;
             float rem = xh;
             for (int q = 0; q < a.npieces; ++q) {
               const __nv_bfloat16 h = __float2bfloat16_rn(rem);
@@ -788,7 +812,7 @@ solve_mixed_v4(SolveArgs a, int64_t n_sys) {
       }
       if (has_obj) {
         // objective at the loss points (FP32 sums of FP32 H rows, FP32 per-point terms)
-        sm.xc[r] = make_float2((float)x.x, (float)x.y);
+        sm.xc[r] = make_float2(xd.x.h, xd.y.h);
         gsync<NM>();
         const int L = a.loss_off[si.s + 1] - a.loss_off[si.s];
         const float* Hl = a.Hl32 + a.t.ln_off[si.s];
@@ -799,11 +823,11 @@ solve_mixed_v4(SolveArgs a, int64_t n_sys) {
         const int64_t wo = a.t.fl_off[si.s] + (int64_t)si.f * L;  // weight / offset base
         const u64* xv = reinterpret_cast<const u64*>(sm.xc);
         const u64* gv = reinterpret_cast<const u64*>(sm.Gs);
-        double lsum = 0.0;
+        df lsum = {0.0f, 0.0f};
         u64 U = 0ull;
         for (int c0 = 0; c0 < a.max_loss; c0 += NM) {
           const int l = c0 + r;
-          cd Gl = {0.0, 0.0};
+          float2 Gl = make_float2(0.0f, 0.0f);
           if (l < L) {
             u64 b0 = 0ull, b1 = 0ull;
             int k = 0;
@@ -819,19 +843,19 @@ solve_mixed_v4(SolveArgs a, int64_t n_sys) {
             float2 bl = make_float2(up(b0).x + up(b1).x, up(b0).y + up(b1).y);
             float wl = 1.0f;
             if (a.loss_offset) {
-              bl.x += (float)a.loss_offset[2 * (wo + l)];
-              bl.y += (float)a.loss_offset[2 * (wo + l) + 1];
+              bl.x += df_from(a.loss_offset[2 * (wo + l)]).h;
+              bl.y += df_from(a.loss_offset[2 * (wo + l) + 1]).h;
             }
             if (a.loss_weight) {
-              wl = (float)a.loss_weight[wo + l];
+              wl = df_from(a.loss_weight[wo + l]).h;
               bl.x *= wl;
               bl.y *= wl;
             }
             float gx, gy;
-            lsum += (double)point_loss_f(a.loss_mode, bl, tb + (int64_t)l * tw, &gx, &gy);
-            Gl = {(double)(gx * wl), (double)(gy * wl)};
+            df_acc(lsum, point_loss_f(a.loss_mode, bl, tb + (int64_t)l * tw, &gx, &gy), 0.0f);
+            Gl = make_float2(gx * wl, -(gy * wl));
           }
-          sm.Gs[r] = make_float2((float)Gl.x, -(float)Gl.y);  // conj(G)
+          sm.Gs[r] = Gl;  // conj(G)
           gsync<NM>();
           if (real_row) {
             const int lc = max(0, min(NM, L - c0));
@@ -842,16 +866,17 @@ solve_mixed_v4(SolveArgs a, int64_t n_sys) {
           }
           gsync<NM>();
         }
-        const double tot = gsum<NM>(lsum, sm, r);
-        if (valid && r == 0) a.loss_part[sys] = tot;
+        const df tot = gsum<NM>(lsum, sm, r);
+        if (valid && r == 0) a.loss_part[sys] = df_double(tot);
         const float2 uf = up(U);
-        u = {(double)uf.x, (double)uf.y};
+        u = {{uf.x, 0.0f}, {uf.y, 0.0f}};
       }
     } else {
       const cd mu = xk;
-      // Im(mu x)/(w C^2) = Im(mu x) w (1/(w C))^2, without a second division
+      // Im(mu x)/(w C^2) = Im(mu x) w (1/(w C))^2, in FP64: the product's range is not FP32's
       if (valid && real_row) {
-        a.grad_part[ioff + r] = (mu.x * x.y + mu.y * x.x) * w * (Dr.y * Dr.y);
+        const double y = df_double(yd);
+        a.grad_part[ioff + r] = (mu.x * x.y + mu.y * x.x) * si.w * (y * y);
         if (!bwd && a.mu_out) {
           a.mu_out[2 * (ioff + r)] = mu.x;
           a.mu_out[2 * (ioff + r) + 1] = mu.y;
