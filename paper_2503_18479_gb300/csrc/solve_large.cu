@@ -13,8 +13,10 @@
 //   U12     the NB pivot rows of the panel over the trailing columns: a unit-lower
 //           triangular solve against the panel's multipliers, a CW-column chunk at a time;
 //   update  every row not chosen yet: A[r][j] -= sum_m L[r][m] U12[m][j]; FP32 register-
-//           tiled (4 listed rows x 4 columns per thread), FP64 thread per column j with
-//           U12[.][j] in registers.
+//           tiled (trailing_update), FP64 thread per column j with U12[.][j] in registers.
+// With 256 or 512 threads in FP32 the trailing columns wait for a block of 32 or 64 columns
+// (large_outer): a panel first takes the products of the block's earlier columns (left-looking)
+// and the trailing matrix is read and written once per block.
 // After the LU the NB x NB diagonal blocks are replaced by their inverses, and the
 // triangular solves run block by block: warp 0 applies the block's inverse, then the other
 // rows take the block's contribution (thread per row), with each step's entries copied a
@@ -92,16 +94,33 @@ struct BlockRed {
   int pidx[2][kLargeMaxWarps];
 };
 
+// Columns of an outer block of the LU: the trailing matrix is read and written once per block
+// instead of once per panel. FP32 with the matrix in the scratch and 256 or 512 threads (more
+// than 128 ports); the others update after every panel.
+template <typename R>
+__host__ __device__ constexpr int large_outer(int T, bool sa) {
+  return sizeof(R) == 4 && !sa && T >= 256 ? (T == 512 ? 64 : 32) : LargeCfg<R>::NB;
+}
+
 // Shared-memory carve-up for systems of up to n ports (host and device agree on it).
 template <typename R>
 struct LargeSmem {
   static constexpr int NB = LargeCfg<R>::NB, CW = LargeCfg<R>::CW;
-  size_t pan, u12, wv, piv, ord, rhs, sv, xk, xc, red, pvec, amat, bytes;
-  __host__ __device__ explicit LargeSmem(int n, bool sa = false) {
+  size_t pan, u12, wv, piv, ord, rhs, sv, xk, xc, red, pvec, lbb, amat, bytes;
+  // T threads per CTA: outer blocks of kb columns (large_outer) keep their U12 chunk and the
+  // warps' multiplier tiles over the panel and U12 regions, and the block's pivot rows over
+  // the FP64 vectors (the panel-by-panel form its multiplier tiles), all idle at that time; the
+  // regions grow where n is too small for that
+  __host__ __device__ explicit LargeSmem(int n, bool sa = false, int T = 128) {
     const size_t cx = sizeof(Cx<R>);
+    const size_t kb = (size_t)large_outer<R>(T, sa);
     size_t o = 0;
     pan = o; o += cx * (size_t)NB * (n + 1);  // panel, column-major, pitch n + 1
     u12 = o; o += cx * (size_t)NB * CW;       // U12 chunk
+    const size_t tiles = (size_t)(T / 32) * 4 * kb * sizeof(float4);  // the warps' multipliers
+    const size_t gemm = kb > NB ? cx * kb * CW + tiles : 0;
+    if (o < gemm) o = gemm;
+    o = (o + 15) / 16 * 16;
     wv = o; o += cx * (size_t)n;              // triangular-solve vector (by row)
     piv = o; o += sizeof(int) * (size_t)n;    // step at which a row became the pivot
     ord = o; o += sizeof(int) * (size_t)n;    // pivot row of each step
@@ -110,6 +129,10 @@ struct LargeSmem {
     sv = o; o += sizeof(cd) * (size_t)n;      // FP64 saved right-hand side
     xk = o; o += sizeof(cd) * (size_t)n;      // FP64 iterate
     xc = o; o += sizeof(cd) * (size_t)n;      // FP64 currents I
+    lbb = rhs;
+    const size_t blk = kb > NB ? cx * kb * (kb + NB) : (sizeof(R) == 4 ? tiles : 0);
+    if (o < lbb + blk) o = lbb + blk;
+    o = (o + 15) / 16 * 16;
     red = o; o += sizeof(BlockRed);
     o = (o + 15) / 16 * 16;
     pvec = o; o += cx * NB;                   // panel part of y or x
@@ -197,6 +220,136 @@ __device__ __forceinline__ void cp_async_elem(Cx<R>* dst, const Cx<R>* src) {
     asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(d), "l"(src) : "memory");
 }
 
+// U rows of an outer block at NC columns from j0: for the block's first nrow pivot rows (a
+// multiple of 16), u = L^-1 a with the block's unit lower triangle lbb ([row][KB]), 16 rows at
+// a time: 16 / RS threads per column take the products with the rows before them, one thread
+// per column the 16-row triangle. Results in ub ([row][NC]) and in the matrix. Every element
+// takes its products in ascending order, as the panel-by-panel update does.
+template <int T, int NC, int KB>
+__device__ inline void outer_u_rows(Cx<float>* __restrict__ A, int N, const int* __restrict__ ord,
+                                    const Cx<float>* __restrict__ lbb, Cx<float>* __restrict__ ub,
+                                    int nrow, int j0) {
+  constexpr int SUB = T / NC < 16 ? T / NC : 16, RS = 16 / SUB;
+  const int tid = threadIdx.x, col = tid % NC, sub = tid / NC;
+  const int j = j0 + col;
+  const bool live = sub < SUB && j < N;
+  Cx<float> v[KB / 16][RS];  // all loads in flight together
+#pragma unroll
+  for (int b = 0; b < KB / 16; ++b)
+#pragma unroll
+    for (int i = 0; i < RS; ++i) {
+      v[b][i] = {0.0f, 0.0f};
+      if (live && 16 * b < nrow) v[b][i] = A[(int64_t)ord[16 * b + sub * RS + i] * N + j];
+    }
+#pragma unroll
+  for (int b = 0; b < KB / 16; ++b) {
+    if (16 * b >= nrow) break;
+    if (sub < SUB) {
+      for (int m = 0; m < 16 * b; ++m) {
+        const Cx<float> u = ub[m * NC + col];
+#pragma unroll
+        for (int i = 0; i < RS; ++i) cx_fnma(v[b][i], lbb[(16 * b + sub * RS + i) * KB + m], u);
+      }
+#pragma unroll
+      for (int i = 0; i < RS; ++i) ub[(16 * b + sub * RS + i) * NC + col] = v[b][i];
+    }
+    __syncthreads();
+    if (sub == 0) {
+      Cx<float> u[16];
+#pragma unroll
+      for (int i = 0; i < 16; ++i) u[i] = ub[(16 * b + i) * NC + col];
+#pragma unroll
+      for (int m = 0; m < 16; ++m)
+#pragma unroll
+        for (int i = m + 1; i < 16; ++i) cx_fnma(u[i], lbb[(16 * b + i) * KB + 16 * b + m], u[m]);
+#pragma unroll
+      for (int i = 0; i < 16; ++i) {
+        ub[(16 * b + i) * NC + col] = u[i];
+        if (j < N) A[(int64_t)ord[16 * b + i] * N + j] = u[i];
+      }
+    }
+    __syncthreads();
+  }
+}
+
+// FP32 trailing update at a chunk of CW columns: a warp takes 4 listed rows x 4 columns a lane
+// (j0 + lane + 32 cc, so that a warp's accesses of one (row, cc) are 256 contiguous bytes) and KB
+// products each, (re, im) in packed registers. Per multiplier l = (a, b) and U12 entry u = (c, d):
+//   v -= l u  <=>  (v.re, v.im) += (b, b) (d, -c) + (-a, -a) (c, d)
+// two fma.rn.f32x2 per complex product (b d first, as cx_fnma). The bound is the FP32 pipe, which
+// takes a packed product every second cycle and leaves the other issue slot for the rest: the
+// multipliers are staged as (-a, -a, b, b), 16 bytes read as one broadcast, because forming
+// those pairs in registers was half of the update's instructions (152 systems of 1024 ports:
+// 4.1e9 of 11.4e9 instructions on the ALU pipe, 46 % of the issue slots used). A tile's
+// multipliers are loaded into registers a tile ahead and put into the warp's own KB x 4 slots
+// of `lst`. src: the multiplier of row r and column m at src[r rs + m ms].
+template <int T, int KB>
+__device__ inline void trailing_update(Cx<float>* __restrict__ A, int N, const int* __restrict__ alist,
+                                       int nact, int j0, const Cx<float>* __restrict__ src, int rs,
+                                       int ms, const Cx<float>* __restrict__ ub, float4* __restrict__ lst) {
+  constexpr int W = T / 32, CW = 128, NL = 4 * KB / 32;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int jc = j0 + lane, ntile = (nact + 3) >> 2;
+  float4* buf = lst + warp * (4 * KB);
+  Cx<float> ln[NL];
+  auto fetch = [&](int t4) {
+#pragma unroll
+    for (int i = 0; i < NL; ++i) {
+      const int e = i * 32 + lane, rr = e / KB, m = e % KB;
+      if (t4 < ntile) ln[i] = src[(int64_t)alist[min(4 * t4 + rr, nact - 1)] * rs + m * ms];
+    }
+  };
+  fetch(warp);
+  for (int t4 = warp; t4 < ntile; t4 += W) {
+    __syncwarp();  // every lane is done with the previous tile's multipliers
+#pragma unroll
+    for (int i = 0; i < NL; ++i) buf[i * 32 + lane] = make_float4(-ln[i].x, -ln[i].x, ln[i].y, ln[i].y);
+    unsigned long long V[4][4];
+#pragma unroll
+    for (int rr = 0; rr < 4; ++rr) {
+      const bool okr = 4 * t4 + rr < nact;
+      const Cx<float>* row = A + (int64_t)alist[okr ? 4 * t4 + rr : 0] * N;
+#pragma unroll
+      for (int cc = 0; cc < 4; ++cc) {
+        const int j = jc + 32 * cc;
+        V[rr][cc] = (okr && j < N) ? *reinterpret_cast<const unsigned long long*>(row + j) : 0ull;
+      }
+    }
+    fetch(t4 + W);
+    __syncwarp();
+#pragma unroll 2
+    for (int m = 0; m < KB; ++m) {
+      ulonglong2 l[4];  // (-a, -a), (b, b)
+#pragma unroll
+      for (int rr = 0; rr < 4; ++rr) l[rr] = *reinterpret_cast<const ulonglong2*>(buf + rr * KB + m);
+      unsigned long long P1[4], P2[4];
+#pragma unroll
+      for (int cc = 0; cc < 4; ++cc) {
+        const Cx<float> u = ub[m * CW + lane + 32 * cc];
+        asm("mov.b64 %0, {%1,%2};" : "=l"(P1[cc]) : "f"(u.x), "f"(u.y));
+        asm("mov.b64 %0, {%1,%2};" : "=l"(P2[cc]) : "f"(u.y), "f"(-u.x));
+      }
+#pragma unroll
+      for (int rr = 0; rr < 4; ++rr)
+#pragma unroll
+        for (int cc = 0; cc < 4; ++cc) {
+          asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(V[rr][cc]) : "l"(l[rr].y), "l"(P2[cc]));
+          asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(V[rr][cc]) : "l"(l[rr].x), "l"(P1[cc]));
+        }
+    }
+#pragma unroll
+    for (int rr = 0; rr < 4; ++rr)
+      if (4 * t4 + rr < nact) {
+        Cx<float>* row = A + (int64_t)alist[4 * t4 + rr] * N;
+#pragma unroll
+        for (int cc = 0; cc < 4; ++cc) {
+          const int j = jc + 32 * cc;
+          if (j < N) *reinterpret_cast<unsigned long long*>(row + j) = V[rr][cc];
+        }
+      }
+  }
+}
+
 // SA: the matrix lives in shared memory (FP32, up to kLargeSmemPorts ports) and goes to the
 // factor scratch only as a copy for the backward; otherwise it stays in the scratch (L2).
 template <typename R, int T, bool SA>
@@ -213,7 +366,7 @@ __global__ void __launch_bounds__(T, T == 128 ? 5 : (T == 256 ? 2 : 1)) solve_la
   if (N <= min_ports) return;  // a register-resident kernel owns this system (CTA-uniform)
 
   extern __shared__ __align__(16) unsigned char dsm[];
-  const LargeSmem<R> L(smem_n, SA);
+  const LargeSmem<R> L(smem_n, SA, T);
   Cx<R>* pan = reinterpret_cast<Cx<R>*>(dsm + L.pan);
   Cx<R>* u12 = reinterpret_cast<Cx<R>*>(dsm + L.u12);
   Cx<R>* wv = reinterpret_cast<Cx<R>*>(dsm + L.wv);
@@ -314,8 +467,15 @@ __global__ void __launch_bounds__(T, T == 128 ? 5 : (T == 256 ? 2 : 1)) solve_la
     __syncthreads();
 
     // ---- blocked LU with partial pivoting ----
+    constexpr int KB = large_outer<R>(T, SA);
+    constexpr bool kOuter = KB > NB;
+    Cx<R>* const lbb = reinterpret_cast<Cx<R>*>(dsm + L.lbb);  // [KB][KB] the block's pivot rows
+    Cx<R>* const upan = lbb + KB * KB;                         // [KB][NB] their U at a panel
     for (int c0 = 0; c0 < N; c0 += NB) {
       const int nb = min(NB, N - c0);
+      const int q0 = kOuter ? c0 % KB : 0;  // columns of the outer block before this panel
+      if constexpr (kOuter)
+        if (q0 > 0) outer_u_rows<T, NB, KB>(A, N, order + (c0 - q0), lbb, upan, q0, c0);
       // eight independent loads in flight per thread (the matrix may be in the scratch)
       for (int e0 = 0; e0 < N * NB; e0 += 8 * T) {
         Cx<R> v[8];
@@ -334,6 +494,32 @@ __global__ void __launch_bounds__(T, T == 128 ? 5 : (T == 256 ? 2 : 1)) solve_la
         }
       }
       __syncthreads();
+      if constexpr (kOuter) {
+        // the products of the outer block's earlier columns, which the trailing update has
+        // not brought yet: a thread per row, its multipliers from the matrix
+        if (q0 > 0) {
+          for (int r = tid; r < N; r += T)
+            if (pivstep[r] == N) {
+              Cx<R> v[NB];
+#pragma unroll
+              for (int j = 0; j < NB; ++j) v[j] = pan[j * NP + r];
+              const Cx<R>* lrow = A + (int64_t)r * N + c0 - q0;
+              for (int m0 = 0; m0 < q0; m0 += 8) {
+                Cx<R> l[8];
+#pragma unroll
+                for (int m = 0; m < 8; ++m) l[m] = lrow[m0 + m];
+#pragma unroll
+                for (int m = 0; m < 8; ++m)
+#pragma unroll
+                  for (int j = 0; j < NB; ++j) cx_fnma(v[j], l[m], upan[(m0 + m) * NB + j]);
+              }
+#pragma unroll
+              for (int j = 0; j < NB; ++j) pan[j * NP + r] = v[j];
+            }
+          // (a row's panel entries are read and written by one thread until the first search
+          // barrier, the loads above are complete)
+        }
+      }
       // pivot steps with one barrier each: a thread reads and writes only its own rows of the
       // panel and their pivot steps, except the pivot row's entries, which its owner last
       // wrote before the barrier of this step's search
@@ -388,6 +574,16 @@ __global__ void __launch_bounds__(T, T == 128 ? 5 : (T == 256 ? 2 : 1)) solve_la
         if (j < nb && pivstep[r] >= c0) A[(int64_t)r * N + c0 + j] = pan[j * NP + r];
       }
       __syncthreads();
+      if constexpr (kOuter) {
+        if (c0 + nb < N) {  // this panel's pivot rows over the block's columns up to it
+          for (int e = tid; e < NB * KB; e += T) {
+            const int i = e / KB, m = e % KB;
+            if (m < q0 + i) lbb[(q0 + i) * KB + m] = A[(int64_t)order[c0 + i] * N + c0 - q0 + m];
+          }
+          __syncthreads();
+        }
+        if (q0 + NB < KB) continue;  // the outer block goes on
+      }
       // FP32: the rows still to be updated (not chosen as pivots yet), listed once per panel
       // in the triangular-solve vector (idle during the LU); warp-aggregated, so the order of
       // the list varies but every row's update is the same
@@ -411,6 +607,15 @@ __global__ void __launch_bounds__(T, T == 128 ? 5 : (T == 256 ? 2 : 1)) solve_la
         }
       }
       // trailing columns, CW at a time
+      if constexpr (kOuter) {
+        Cx<R>* const ub = pan;               // [KB][CW], over the panel (in the matrix by now)
+        float4* const lst = reinterpret_cast<float4*>(ub + KB * CW);  // the warps' multipliers
+        for (int j0 = c0 + nb; j0 < N; j0 += CW) {
+          outer_u_rows<T, CW, KB>(A, N, order + (c0 - q0), lbb, ub, KB, j0);
+          trailing_update<T, KB>(A, N, alist, nact, j0, A + c0 - q0, N, 1, ub, lst);
+          __syncthreads();
+        }
+      } else
       for (int j0 = c0 + nb; j0 < N; j0 += CW) {
         if (tid < CW) {
           const int j = j0 + tid;
@@ -440,66 +645,8 @@ __global__ void __launch_bounds__(T, T == 128 ? 5 : (T == 256 ? 2 : 1)) solve_la
         }
         __syncthreads();
         if constexpr (kF) {
-          // register-tiled update: a thread takes 4 listed rows x 4 columns (j0 + lane + 32 cc,
-          // so that a warp's loads of one (row, cc) are 256 contiguous bytes: conflict-free in
-          // shared memory, coalesced in the scratch),
-          // the (re, im) pairs of a tile in packed registers; per panel column m, with the
-          // multiplier l = (a, b) and the U12 entry u = (c, d):
-          //   v -= l u  <=>  (v.re, v.im) += (b, b) (d, -c) + (-a, -a) (c, d)
-          // two fma.rn.f32x2 per complex multiply-add, 8 shared loads per 16 of them
-          const int jc = j0 + lane;  // the warp covers the chunk's 128 columns
-          const int ntile = (nact + 3) >> 2;
-          for (int t4 = warp; t4 < ntile; t4 += W) {
-            int rw[4];
-            bool okr[4];
-#pragma unroll
-            for (int rr = 0; rr < 4; ++rr) {
-              okr[rr] = 4 * t4 + rr < nact;
-              rw[rr] = alist[okr[rr] ? 4 * t4 + rr : 0];
-            }
-            unsigned long long V[4][4];
-#pragma unroll
-            for (int rr = 0; rr < 4; ++rr)
-#pragma unroll
-              for (int cc = 0; cc < 4; ++cc) {
-                const int j = jc + 32 * cc;
-                V[rr][cc] = (okr[rr] && j < N)
-                                ? *reinterpret_cast<const unsigned long long*>(A + (int64_t)rw[rr] * N + j)
-                                : 0ull;
-              }
-#pragma unroll 2
-            for (int m = 0; m < NB; ++m) {
-              unsigned long long LA[4], LB[4], P1[4], P2[4];
-#pragma unroll
-              for (int rr = 0; rr < 4; ++rr) {
-                const Cx<R> l = pan[m * NP + rw[rr]];
-                asm("mov.b64 %0, {%1,%1};" : "=l"(LA[rr]) : "f"(-l.x));
-                asm("mov.b64 %0, {%1,%1};" : "=l"(LB[rr]) : "f"(l.y));
-              }
-#pragma unroll
-              for (int cc = 0; cc < 4; ++cc) {
-                const Cx<R> u = u12[m * CW + lane + 32 * cc];
-                asm("mov.b64 %0, {%1,%2};" : "=l"(P1[cc]) : "f"(u.x), "f"(u.y));
-                asm("mov.b64 %0, {%1,%2};" : "=l"(P2[cc]) : "f"(u.y), "f"(-u.x));
-              }
-#pragma unroll
-              for (int rr = 0; rr < 4; ++rr)
-#pragma unroll
-                for (int cc = 0; cc < 4; ++cc) {
-                  // the order of cx_fnma (b d first): the same roundings as the per-column form
-                  asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(V[rr][cc]) : "l"(LB[rr]), "l"(P2[cc]));
-                  asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(V[rr][cc]) : "l"(LA[rr]), "l"(P1[cc]));
-                }
-            }
-#pragma unroll
-            for (int rr = 0; rr < 4; ++rr)
-#pragma unroll
-              for (int cc = 0; cc < 4; ++cc) {
-                const int j = jc + 32 * cc;
-                if (okr[rr] && j < N)
-                  *reinterpret_cast<unsigned long long*>(A + (int64_t)rw[rr] * N + j) = V[rr][cc];
-              }
-          }
+          trailing_update<T, NB>(A, N, alist, nact, j0, pan, 1, NP, u12,
+                                 reinterpret_cast<float4*>(dsm + L.lbb));
         } else {
           {
             const int col = tid % CW, rg = tid / CW;
@@ -982,13 +1129,14 @@ static bool large_in_smem(mts_precision prec, int T, int max_ports) {
 
 size_t large_solve_smem(mts_precision prec, int max_ports) {
   if (prec == MTS_FP64) return LargeSmem<double>(max_ports).bytes;
-  return LargeSmem<float>(max_ports, large_in_smem(prec, large_threads(max_ports), max_ports)).bytes;
+  const int T = large_threads(max_ports);
+  return LargeSmem<float>(max_ports, large_in_smem(prec, T, max_ports), T).bytes;
 }
 
 template <typename R, int T, bool SA>
 static cudaError_t launch_large(const SolveArgs& a, int64_t n_sys, int min_ports, int max_ports,
                                 void* scratch, cudaStream_t st) {
-  const size_t sm = LargeSmem<R>(max_ports, SA).bytes;
+  const size_t sm = LargeSmem<R>(max_ports, SA, T).bytes;
   cudaError_t e = cudaFuncSetAttribute(solve_large_kernel<R, T, SA>,
                                        cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
   if (e != cudaSuccess) return e;
