@@ -350,10 +350,19 @@ __device__ inline void trailing_update(Cx<float>* __restrict__ A, int N, const i
   }
 }
 
+// the same for 16 aligned bytes
+template <typename R>
+__device__ __forceinline__ void cp_async16(Cx<R>* dst, const Cx<R>* src) {
+  const uint32_t d = (uint32_t)__cvta_generic_to_shared(dst);
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(d), "l"(src) : "memory");
+}
+
 // SA: the matrix lives in shared memory (FP32, up to kLargeSmemPorts ports) and goes to the
 // factor scratch only as a copy for the backward; otherwise it stays in the scratch (L2).
+// Four CTAs of 128 threads per SM (128 registers): five (96 registers) took 577 against 484 us for
+// 1000 systems of 72 ports and 675 against 585 us for 96, and 3373 against 3477 us for 4000 of 128.
 template <typename R, int T, bool SA>
-__global__ void __launch_bounds__(T, T == 128 ? 5 : (T == 256 ? 2 : 1)) solve_large_kernel(SolveArgs a, int64_t n_sys,
+__global__ void __launch_bounds__(T, T == 128 ? 4 : (T == 256 ? 2 : 1)) solve_large_kernel(SolveArgs a, int64_t n_sys,
                                                                      int min_ports, int smem_n,
                                                                      Cx<R>* __restrict__ scratch) {
   constexpr int NB = LargeCfg<R>::NB, CW = LargeCfg<R>::CW;
@@ -497,6 +506,7 @@ __global__ void __launch_bounds__(T, T == 128 ? 5 : (T == 256 ? 2 : 1)) solve_la
       if constexpr (kOuter) {
         // the products of the outer block's earlier columns, which the trailing update has
         // not brought yet: a thread per row, its multipliers from the matrix
+        const bool row16 = (N & 1) == 0 && (reinterpret_cast<uintptr_t>(A) & 15) == 0;
         if (q0 > 0) {
           for (int r = tid; r < N; r += T)
             if (pivstep[r] == N) {
@@ -505,9 +515,15 @@ __global__ void __launch_bounds__(T, T == 128 ? 5 : (T == 256 ? 2 : 1)) solve_la
               for (int j = 0; j < NB; ++j) v[j] = pan[j * NP + r];
               const Cx<R>* lrow = A + (int64_t)r * N + c0 - q0;
               for (int m0 = 0; m0 < q0; m0 += 8) {
-                Cx<R> l[8];
+                alignas(16) Cx<R> l[8];
+                if (row16) {
 #pragma unroll
-                for (int m = 0; m < 8; ++m) l[m] = lrow[m0 + m];
+                  for (int m = 0; m < 8; m += 2)
+                    *reinterpret_cast<float4*>(l + m) = *reinterpret_cast<const float4*>(lrow + m0 + m);
+                } else {
+#pragma unroll
+                  for (int m = 0; m < 8; ++m) l[m] = lrow[m0 + m];
+                }
 #pragma unroll
                 for (int m = 0; m < 8; ++m)
 #pragma unroll
@@ -763,12 +779,17 @@ __global__ void __launch_bounds__(T, T == 128 ? 5 : (T == 256 ? 2 : 1)) solve_la
   // ---- solve A x = rhs (FP64 rhs in shared memory) into wv (by row) with the factors;
   // the unknown of column k ends in wv[order[k]]. With the factors in the scratch, each
   // step's entries are copied one step ahead (cp.async) into shared memory that is idle
-  // during the solves: the blocks of the thread's rows that the row update needs (in the
-  // panel region, element m of row r at m N + r) and warp 0's rows of the diagonal block (in
-  // the U12 region), so that their latency overlaps the barrier and the diagonal block's
-  // products. A thread reads only what it copied. ----
-  Cx<R>* const stg = pan;  // [NB][N]
+  // during the solves, so that their latency overlaps the barrier and the diagonal block's
+  // products: in the panel region the 128 bytes of each row that the row update needs, and in
+  // the U12 region warp 0's rows of the diagonal block. A warp copies the rows of its own
+  // threads (no other warp reads them), eight lanes a row in 16-byte units, unit u of row r at
+  // u ^ (r % 8) so that threads of consecutive rows read different banks. Copies of one entry
+  // per lane and row fetched every 32-byte sector four times. ----
+  Cx<R>* const stg = pan;  // [N][128 bytes]
   Cx<R>* const dstg = u12;  // [NB][32]
+  constexpr int UE = 16 / (int)sizeof(Cx<R>);  // entries of a 16-byte unit
+  const bool unit16 = (N & 1) == 0 && (reinterpret_cast<uintptr_t>(A) & 15) == 0;
+  auto stg_at = [&](int r, int m) -> Cx<R>* { return stg + r * NB + ((m / UE) ^ (r & 7)) * UE + m % UE; };
   auto lu_solve = [&]() {
     for (int r = tid; r < N; r += T) wv[r] = {(R)rhs[r].x, (R)rhs[r].y};
     const int last = (N - 1) / NB * NB;
@@ -776,12 +797,23 @@ __global__ void __launch_bounds__(T, T == 128 ? 5 : (T == 256 ? 2 : 1)) solve_la
     auto fetch = [&](int c0, bool fwd) {
       if constexpr (!SA) {
         const int nb = min(NB, N - c0);
-        for (int r = tid; r < N; r += T)
-          if (fwd ? pivstep[r] >= c0 + nb : pivstep[r] < c0) {
+        __syncwarp();  // the warp's rows of the previous step have been read
+        for (int rb = warp * 32; rb < N; rb += T) {
+          if (sizeof(R) == 8 || (unit16 && nb == NB)) {
 #pragma unroll
-            for (int m = 0; m < NB; ++m)
-              if (m < nb) cp_async_elem(stg + m * N + r, A + (int64_t)r * N + c0 + m);
+            for (int i = 0; i < 8; ++i) {
+              const int r = rb + i * 4 + (lane >> 3), u = lane & 7;
+              if (r < N && (fwd ? pivstep[r] >= c0 + nb : pivstep[r] < c0) && (sizeof(R) == 4 || u < nb))
+                cp_async16(stg_at(r, u * UE), A + (int64_t)r * N + c0 + u * UE);
+            }
+          } else {
+            for (int i = 0; i < 16; ++i) {
+              const int r = rb + i * 2 + (lane >> 4), m = lane & 15;
+              if (r < N && m < nb && (fwd ? pivstep[r] >= c0 + nb : pivstep[r] < c0))
+                cp_async_elem(stg_at(r, m), A + (int64_t)r * N + c0 + m);
+            }
           }
+        }
         if (warp == 0 && lane < nb) {
           const int pi = order[c0 + lane];
 #pragma unroll
@@ -792,12 +824,26 @@ __global__ void __launch_bounds__(T, T == 128 ? 5 : (T == 256 ? 2 : 1)) solve_la
         asm volatile("cp.async.commit_group;" ::: "memory");
       }
     };
-    // entry m of the staged block of row r / of this lane's diagonal row (the matrix itself
-    // when it is in shared memory)
-    auto row_elem = [&](int r, int c0, int m) -> Cx<R> {
-      if constexpr (SA) return A[(int64_t)r * N + c0 + m];
-      else return stg[m * N + r];
+    // this thread's rows take the block's contribution, products in ascending order
+    auto row_update = [&](int r, int c0, int nb) {
+      Cx<R> v = wv[r];
+      if constexpr (SA) {
+#pragma unroll
+        for (int m = 0; m < NB; ++m)
+          if (m < nb) cx_fnma(v, A[(int64_t)r * N + c0 + m], pvec[m]);
+      } else {
+#pragma unroll
+        for (int u = 0; u < 8; ++u) {
+          alignas(16) Cx<R> e[UE];
+          *reinterpret_cast<uint4*>(e) = *reinterpret_cast<const uint4*>(stg_at(r, u * UE));
+#pragma unroll
+          for (int q = 0; q < UE; ++q)
+            if (u * UE + q < nb) cx_fnma(v, e[q], pvec[u * UE + q]);
+        }
+      }
+      wv[r] = v;
     };
+    // entry m of this lane's diagonal row (the matrix itself when it is in shared memory)
     auto diag_elem = [&](int c0, int pi, int m) -> Cx<R> {
       if constexpr (SA) return A[(int64_t)pi * N + c0 + m];
       else return dstg[m * 32 + lane];
@@ -830,14 +876,9 @@ __global__ void __launch_bounds__(T, T == 128 ? 5 : (T == 256 ? 2 : 1)) solve_la
       }
       __syncthreads();
       if constexpr (!SA) asm volatile("cp.async.wait_all;" ::: "memory");
+      __syncwarp();  // the warp's copies, by whichever of its lanes
       for (int r = tid; r < N; r += T)
-        if (pivstep[r] >= c0 + nb) {
-          Cx<R> v = wv[r];
-#pragma unroll
-          for (int m = 0; m < NB; ++m)
-            if (m < nb) cx_fnma(v, row_elem(r, c0, m), pvec[m]);
-          wv[r] = v;
-        }
+        if (pivstep[r] >= c0 + nb) row_update(r, c0, nb);
       if (c0 + NB < N) fetch(c0 + NB, true);
       else fetch(last, false);
       __syncthreads();
@@ -869,14 +910,9 @@ __global__ void __launch_bounds__(T, T == 128 ? 5 : (T == 256 ? 2 : 1)) solve_la
       }
       __syncthreads();
       if constexpr (!SA) asm volatile("cp.async.wait_all;" ::: "memory");
+      __syncwarp();
       for (int r = tid; r < N; r += T)
-        if (pivstep[r] < c0) {
-          Cx<R> v = wv[r];
-#pragma unroll
-          for (int m = 0; m < NB; ++m)
-            if (m < nb) cx_fnma(v, row_elem(r, c0, m), pvec[m]);
-          wv[r] = v;
-        }
+        if (pivstep[r] < c0) row_update(r, c0, nb);
       if (c0 > 0) fetch(c0 - NB, false);
       __syncthreads();
     }
