@@ -23,30 +23,48 @@
 namespace mts {
 
 // ---------------------------------------------------------------------------------------
-// FP64 kernel: G groups of NM threads per CTA, rows in dynamic shared memory.
+// FP64 kernel: groups of NM threads, rows in dynamic shared memory; one group per CTA for
+// NM = 64 (three systems of 67 KB on an SM), several per 128-thread CTA below.
+//
+// The bound is the FP64 pipe (a warp's instruction holds it for 16 cycles): about 21,000 of its
+// instructions a 64-port system, 16,000 of them the LU's updates. Everything else on a pivot step
+// is kept off that pipe or shared: the pivot search runs on the high words of |a|^2 (20 bits of
+// mantissa decide, which row of nearly equal ones is taken does not matter) with the row in the
+// low bits, by one redux; a step divides once, by |pivot|^2, and keeps the inverse pivot on the
+// diagonal for the solves; one barrier a step, because a chosen row is never written again and
+// the search words alternate by step parity. 1024 systems of 64 ports with objective and
+// adjoint: 3030 us with two divisions a row and step, FP64 compares and three barriers.
 // ---------------------------------------------------------------------------------------
 template <int NM>
 struct Fp64Smem {
+  static constexpr int CT = NM >= 64 ? NM : 128;  // threads of a CTA
   static constexpr int P = NM + 1;  // row pitch (complex) to spread banks
   static constexpr size_t per_group =
-      sizeof(cd) * (size_t)NM * P + sizeof(cd) * NM /* rhs */ + sizeof(cd) * NM /* xs */ +
-      sizeof(cd) * NM /* G */ + sizeof(double) * 32 /* red */ + sizeof(int) * 32;
+      sizeof(cd) * (size_t)NM * P + sizeof(cd) * NM /* xs */ + sizeof(cd) * NM /* G */ +
+      sizeof(double) * 32 /* red */ + sizeof(int) * 32;
 };
 
 template <int NM>
-__global__ void __launch_bounds__(NM >= 128 ? NM : 128) solve_fp64_kernel(SolveArgs a, int64_t n_sys) {
-  constexpr int CT = NM >= 128 ? NM : 128;
+__device__ __forceinline__ void fp64_sync() {
+  if constexpr (NM <= 32) __syncwarp();
+  else __syncthreads();
+}
+
+template <int NM>
+__global__ void __launch_bounds__(Fp64Smem<NM>::CT) solve_fp64_kernel(SolveArgs a, int64_t n_sys) {
+  constexpr int CT = Fp64Smem<NM>::CT;
   constexpr int G = CT / NM;
   constexpr int P = Fp64Smem<NM>::P;
+  constexpr int NW = NM > 32 ? NM / 32 : 1;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int grp = threadIdx.x / NM, r = threadIdx.x % NM;
   unsigned char* base = smem_raw + grp * Fp64Smem<NM>::per_group;
   cd* A = reinterpret_cast<cd*>(base);
-  cd* rhs = A + NM * P;
-  cd* xs = rhs + NM;
+  cd* xs = A + NM * P;
   cd* Gs = xs + NM;
   double* red = reinterpret_cast<double*>(Gs + NM);
   int* redi = reinterpret_cast<int*>(red + 32);
+  unsigned* ukey = reinterpret_cast<unsigned*>(redi);  // [2][NW] pivot search by step parity
 
   const int64_t li = (int64_t)blockIdx.x * G + grp;
   const bool in_range = li < n_sys;
@@ -59,10 +77,12 @@ __global__ void __launch_bounds__(NM >= 128 ? NM : 128) solve_fp64_kernel(SolveA
   const bool real_row = r < N;
   double Cr = real_row ? a.C[si.b * a.n_ports + si.k0 + r] : 1.0;
   const double* Ms = a.M64 + a.t.nn_off[si.s];
-  // assemble row r (Eq. 2, 11): A_rj = j w M_rj, A_rr += R_r + 1/(j w C_r)
+  // assemble row r (Eq. 2, 11): A_rj = j w M_rj, A_rr += R_r + 1/(j w C_r); M is symmetric, so
+  // row r is read as column r (consecutive threads, consecutive values)
+#pragma unroll 8
   for (int j = 0; j < NM; ++j) {
     cd v = {0.0, 0.0};
-    if (real_row && j < N) v.y = w * Ms[r * N + j];
+    if (real_row && j < N) v.y = w * Ms[j * N + r];
     A[r * P + j] = v;
   }
   if (real_row) {
@@ -78,65 +98,95 @@ __global__ void __launch_bounds__(NM >= 128 ? NM : 128) solve_fp64_kernel(SolveA
     const double* Vp = a.V + 2 * (a.t.fn_off[si.s] + (int64_t)si.f * N + r);
     v0 = {Vp[0], Vp[1]};
   }
-  rhs[r] = v0;
-  __syncthreads();
 
   // ---- LU with partial pivoting (rows stay in place) ----
   int pivstep = NM;  // step at which this row became the pivot
   for (int k = 0; k < NM; ++k) {
-    double key = (pivstep < NM) ? -1.0 : cabs2(A[r * P + k]);
-    if (!(key >= -1.0)) key = 0.0;  // NaN: still a candidate, never below a chosen row
-    int idx = r;
-    if (NM <= 32) {
-      argmax_shfl_d(key, idx, NM);
+    const cd cur = A[r * P + k];
+    // |a|^2's high word; chosen rows 0; NaN ranks lowest of the candidates
+    unsigned key = 0u;
+    if (pivstep == NM) {
+      key = (unsigned)__double2hiint(cabs2(cur));
+      if (key > 0x7ff00000u) key = 0u;
+      key = (key & ~127u) | 64u | (unsigned)(63 - r);
+    }
+    int p;
+    if constexpr (NM < 32) {
+#pragma unroll
+      for (int o = NM >> 1; o > 0; o >>= 1) key = max(key, __shfl_xor_sync(0xffffffffu, key, o, NM));
     } else {
-      argmax_shfl_d(key, idx, 32);
-      if ((r & 31) == 0) {
-        red[r >> 5] = key;
-        redi[r >> 5] = idx;
-      }
+      unsigned m;
+      asm volatile("redux.sync.max.u32 %0, %1, 0xffffffff;" : "=r"(m) : "r"(key));
+      key = m;
+    }
+    if constexpr (NW > 1) {
+      unsigned* uk = ukey + (k & 1) * NW;
+      if ((r & 31) == 0) uk[r >> 5] = key;
       __syncthreads();
-      key = red[0];
-      idx = redi[0];
-      for (int q = 1; q < NM / 32; ++q)
-        if (red[q] > key || (red[q] == key && redi[q] < idx)) {
-          key = red[q];
-          idx = redi[q];
-        }
+      key = uk[0];
+#pragma unroll
+      for (int q = 1; q < NW; ++q) key = max(key, uk[q]);
+    } else {
+      __syncwarp();  // every row's update of the last step in place
     }
-    const int p = idx;
-    if (r == p) pivstep = k;
-    __syncthreads();
-    if (pivstep > k) {
-      cd l = cdiv(A[r * P + k], A[p * P + k]);
+    p = 63 - (int)(key & 63u);
+    const cd piv = A[p * P + k];
+    const double dinv = 1.0 / cabs2(piv);
+    const cd inv = {piv.x * dinv, -piv.y * dinv};
+    if (r == p) {
+      pivstep = k;
+    } else if (pivstep == NM) {
+      const cd l = cmul(cur, inv);
       A[r * P + k] = l;
-      for (int j = k + 1; j < NM; ++j) A[r * P + j] = csub(A[r * P + j], cmul(l, A[p * P + j]));
+#pragma unroll 4
+      for (int j = k + 1; j < NM; ++j) {
+        const cd u = A[p * P + j];
+        cd v = A[r * P + j];
+        v.x = fma(-l.x, u.x, fma(l.y, u.y, v.x));
+        v.y = fma(-l.x, u.y, fma(-l.y, u.x, v.y));
+        A[r * P + j] = v;
+      }
     }
-    __syncthreads();
+  }
+  // the inverse pivots replace the diagonal (nobody reads another row's own pivot from here)
+  fp64_sync<NM>();
+  {
+    const cd piv = A[r * P + pivstep];
+    const double dinv = 1.0 / cabs2(piv);
+    A[r * P + pivstep] = {piv.x * dinv, -piv.y * dinv};
   }
 
-  // triangular solves on rhs (forward with the multipliers, then back with U)
-  auto solve_inplace = [&](cd myrhs) -> cd {
+  // triangular solves on rhs (forward with the multipliers, then back with U); a step's unknown
+  // has its own slot, so one barrier a step
+  auto solve_inplace = [&](cd b) -> cd {
     // forward: L y = P b
     for (int k = 0; k < NM; ++k) {
-      if (pivstep == k) xs[k] = myrhs;
-      __syncthreads();
-      if (pivstep > k) myrhs = csub(myrhs, cmul(A[r * P + k], xs[k]));
-      __syncthreads();
+      if (pivstep == k) xs[k] = b;
+      fp64_sync<NM>();
+      if (pivstep > k) {
+        const cd l = A[r * P + k], y = xs[k];
+        b.x = fma(-l.x, y.x, fma(l.y, y.y, b.x));
+        b.y = fma(-l.x, y.y, fma(-l.y, y.x, b.y));
+      }
     }
+    fp64_sync<NM>();
     // back: U x = y
     for (int k = NM - 1; k >= 0; --k) {
-      if (pivstep == k) xs[k] = cdiv(myrhs, A[r * P + k]);
-      __syncthreads();
-      if (pivstep < k) myrhs = csub(myrhs, cmul(A[r * P + k], xs[k]));
+      if (pivstep == k) xs[k] = cmul(b, A[r * P + k]);
+      fp64_sync<NM>();
+      if (pivstep < k) {
+        const cd u = A[r * P + k], y = xs[k];
+        b.x = fma(-u.x, y.x, fma(u.y, y.y, b.x));
+        b.y = fma(-u.x, y.y, fma(-u.y, y.x, b.y));
+      }
     }
-    __syncthreads();
+    fp64_sync<NM>();
     return xs[r];
   };
 
   cd x = {0.0, 0.0};
   if (!bwd) {
-    x = solve_inplace(rhs[r]);
+    x = solve_inplace(v0);
   } else if (real_row) {
     const double* Ip = a.I + 2 * (ioff + r);
     x = {Ip[0], Ip[1]};
@@ -151,9 +201,9 @@ __global__ void __launch_bounds__(NM >= 128 ? NM : 128) solve_fp64_kernel(SolveA
     }
   }
   bool bad = !(isfinite(x.x) && isfinite(x.y)) && real_row;
-  __syncthreads();
+  fp64_sync<NM>();
   xs[r] = x;  // currents visible to the whole group
-  __syncthreads();
+  fp64_sync<NM>();
 
   // ---- objective and adjoint right-hand side ----
   bool do_adj = bwd || a.target != nullptr;
@@ -191,7 +241,7 @@ __global__ void __launch_bounds__(NM >= 128 ? NM : 128) solve_fp64_kernel(SolveA
         Gl.y *= wl;
       }
       Gs[r] = Gl;
-      __syncthreads();
+      fp64_sync<NM>();
       if (real_row) {
         int lc = max(0, min(NM, L - c0));
         for (int q = 0; q < lc; ++q) {
@@ -200,7 +250,7 @@ __global__ void __launch_bounds__(NM >= 128 ? NM : 128) solve_fp64_kernel(SolveA
           u.y -= h * Gs[q].y;  // conj(G)
         }
       }
-      __syncthreads();
+      fp64_sync<NM>();
     }
   } else if (bwd && real_row) {
     const double* up = a.rhs_in + 2 * (ioff + r);
@@ -214,9 +264,9 @@ __global__ void __launch_bounds__(NM >= 128 ? NM : 128) solve_fp64_kernel(SolveA
       if (r == 0 && valid) a.loss_part[sys] = v;
     } else {
       for (int off = 16; off > 0; off >>= 1) v += __shfl_xor_sync(0xffffffffu, v, off);
-      __syncthreads();
+      fp64_sync<NM>();
       if ((r & 31) == 0) red[r >> 5] = v;
-      __syncthreads();
+      fp64_sync<NM>();
       if (r == 0) {
         double tot = 0.0;
         for (int q = 0; q < NM / 32; ++q) tot += red[q];
@@ -237,11 +287,11 @@ __global__ void __launch_bounds__(NM >= 128 ? NM : 128) solve_fp64_kernel(SolveA
   }
   // status
   // non-finite flag of this group's system only (a CTA holds G systems)
-  __syncthreads();
+  fp64_sync<NM>();
   if (r == 0) redi[0] = 0;
-  __syncthreads();
+  fp64_sync<NM>();
   if (bad) redi[0] = 1;
-  __syncthreads();
+  fp64_sync<NM>();
   if (valid && r == 0 && !bwd) a.status[sys] = redi[0] ? 2 : 0;
 }
 
@@ -285,7 +335,7 @@ __global__ void reduce_kernel(ReduceArgs a) {
 // ---------------------------------------------------------------------------------------
 template <int NM>
 static cudaError_t launch_fp64(const SolveArgs& a, int64_t n_sys, cudaStream_t st) {
-  constexpr int CT = NM >= 128 ? NM : 128;
+  constexpr int CT = Fp64Smem<NM>::CT;
   constexpr int G = CT / NM;
   size_t smem = Fp64Smem<NM>::per_group * G;
   cudaError_t e = cudaFuncSetAttribute(solve_fp64_kernel<NM>,
