@@ -19,6 +19,7 @@ BUILD = os.path.join(HERE, "_build")
 LIBDIR = os.path.join(HERE, "lib")
 LIB = os.path.join(LIBDIR, "libmts.so")
 SOURCES = ["abi.cu", "basis.cu", "solve.cu", "solve_mixed.cu", "solve_large.cu", "superpose.cu", "superpose_tc.cu",
+           "superpose_fp64_tc.cu",
            "backward.cu",
            "static_solve.cu", "optim.cu", "sroute.cu", "field_adjoint_tc.cu"]
 HEADERS = ["common.cuh", "kernels.h", "solve_common.cuh", "tc_common.cuh"]

@@ -335,7 +335,17 @@ cudaError_t superpose_core(const mts_problem* pb, mts_precision prec, const void
   a.npieces = n_pieces(prec);
   a.B_out = B_out;
   a.err = err;
-  if (pb->n_struct == 1 && a.total_units > 0) {
+  // FP64, one structure: the tensor cores where their tiles are the faster form
+  int64_t units64 = 0;
+  int sms = 0;
+  if (pb->n_struct == 1 && prec == MTS_FP64 && a.total_simt > 0) {
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms <= 0)
+      sms = 1;
+    units64 = superpose_fp64_tc_units(pb->h_port_off[1], pb->h_point_off[1], n_cfg * pb->h_freq_off[1], sms);
+  }
+  if (pb->n_struct == 1 && (a.total_units > 0 || units64 > 0)) {
     a.uni.on = 1;
     a.uni.N = pb->h_port_off[1];
     a.uni.F = pb->h_freq_off[1];
@@ -344,6 +354,7 @@ cudaError_t superpose_core(const mts_problem* pb, mts_precision prec, const void
     a.uni.nptile = (a.uni.P + kTileP - 1) / kTileP;
     a.uni.nntile = (2 * n_cfg * a.uni.F + kTileN - 1) / kTileN;
   }
+  if (units64 > 0) return launch_superpose_fp64_tc(a, units64, sms, st);
   return launch_superpose(a, prec, st);
 }
 

@@ -116,6 +116,12 @@ struct UniformUnits {
   int64_t P, nptile, nntile;
 };
 
+struct SuperposeArgs;
+// FP64 superposition of one structure on the tensor cores (superpose_fp64_tc.cu): its work
+// units, 0 where the SIMT kernel is faster.
+int64_t superpose_fp64_tc_units(int64_t N, int64_t P, int64_t nsys, int sms);
+cudaError_t launch_superpose_fp64_tc(const SuperposeArgs& a, int64_t units, int sms, cudaStream_t st);
+
 struct SuperposeArgs {
   int n_struct, n_freq, n_ports;
   const int32_t* port_off;
