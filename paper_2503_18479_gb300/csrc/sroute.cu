@@ -201,65 +201,157 @@ __device__ double2 sr_df_dot(const float2* __restrict__ Mh, const float2* __rest
   return make_double2((double)rh + (double)rl, (double)ih + (double)il);
 }
 
-// LU with partial pivoting of the n x n matrix a (row-major, shared memory), in place:
+// c -= a b (complex)
+template <typename V>
+__device__ __forceinline__ void sr_fnma(V& c, V a, V b) {
+  c.x = fma(-a.x, b.x, fma(a.y, b.y, c.x));
+  c.y = fma(-a.x, b.y, fma(-a.y, b.x, c.y));
+}
+
+// The warp's largest key and the smallest lane that holds it; key < 0 marks rows out of the search.
+__device__ inline int sr_warp_argmax(float key, float* best) {
+  // non-negative floats order as their bits; 0 is "none"
+  const unsigned b = key >= 0.0f ? __float_as_uint(key) + 1u : 0u;
+  unsigned m;
+  asm volatile("redux.sync.max.u32 %0, %1, 0xffffffff;" : "=r"(m) : "r"(b));
+  *best = m ? __uint_as_float(m - 1u) : -1.0f;
+  return __ffs(__ballot_sync(0xffffffffu, b == m)) - 1;
+}
+__device__ inline int sr_warp_argmax(double key, double* best) {
+  double m = key;
+  for (int o = 16; o > 0; o >>= 1) m = fmax(m, __shfl_xor_sync(0xffffffffu, m, o));
+  *best = m;
+  return __ffs(__ballot_sync(0xffffffffu, key == m)) - 1;
+}
+
+// LU with partial pivoting of the n x n matrix a (row-major, shared memory, n <= 96), in place:
 // P a = L U, unit L below the diagonal. perm[i] = the original row now at row i. The pivot
 // is the first row of largest |a_ik|^2 (a NaN candidate ranks as 0). Returns 1 on a zero
 // (or non-finite) pivot.
+//
+// The kernel is bound by issued instructions, most of them this factorisation's when every step
+// updated the whole trailing matrix from shared memory (about 116,000 of 190,000 warp
+// instructions per 65-port system, four barriers a step). So panels of eight columns: a thread
+// holds its row's eight entries in registers through the panel's pivot steps (one barrier each:
+// every warp publishes its candidate row, the search words alternate by step parity), the
+// chosen rows are then exchanged into place (a thread per column), and the trailing matrix takes
+// one update of eight products, a thread per column and group of rows.
+constexpr int kSrPanel = 8;
+static_assert(kSrMaxN0 <= kSrThreads, "a thread per row");
+
 template <typename LT>
-__device__ int sr_factor(int n, typename SrT<LT>::V* a, int* perm, int* s_int) {
+__device__ int sr_factor(int n, typename SrT<LT>::V* a, int* perm) {
   using V = typename SrT<LT>::V;
+  constexpr int PB = kSrPanel;
+  __shared__ V s_cand[2][kSrWarps][PB];
+  __shared__ LT s_key[2][kSrWarps];
+  __shared__ int s_idx[2][kSrWarps], s_piv[PB];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   for (int i = tid; i < n; i += kSrThreads) perm[i] = i;
-  __syncthreads();
   int bad = 0;
-  for (int k = 0; k < n; ++k) {
-    if (warp == 0) {
-      LT best = (LT)-1;
-      int bi = n;
-      for (int i = k + lane; i < n; i += 32) {
-        const V v = a[i * n + k];
-        LT m = v.x * v.x + v.y * v.y;
-        if (!(m == m)) m = (LT)0;
-        if (m > best) {
-          best = m;
-          bi = i;
+  for (int c0 = 0; c0 < n; c0 += PB) {
+    const int nb = min(PB, n - c0);
+    bool open = tid >= c0 && tid < n;  // this thread's row is in the search
+    const bool own = open;
+    V v[PB];
+#pragma unroll
+    for (int j = 0; j < PB; ++j) v[j] = own && j < nb ? a[tid * n + c0 + j] : V{0, 0};
+#pragma unroll
+    for (int kk = 0; kk < PB; ++kk) {
+      if (kk < nb) {
+        const int buf = kk & 1;
+        LT key = (LT)-1;
+        if (open) {
+          key = v[kk].x * v[kk].x + v[kk].y * v[kk].y;
+          if (!(key == key)) key = (LT)0;
         }
-      }
-      for (int o = 16; o > 0; o >>= 1) {
-        const LT ob = __shfl_down_sync(0xffffffffu, best, o);
-        const int oi = __shfl_down_sync(0xffffffffu, bi, o);
-        if (ob > best || (ob == best && oi < bi)) {
-          best = ob;
-          bi = oi;
+        LT wbest;
+        const int wl = sr_warp_argmax(key, &wbest);
+        if (lane == wl) {
+          s_key[buf][warp] = wbest;
+          s_idx[buf][warp] = tid;
+#pragma unroll
+          for (int j = kk; j < PB; ++j) s_cand[buf][warp][j] = v[j];
         }
-      }
-      if (lane == 0) {
-        s_int[0] = bi;
-        s_int[1] = !(best > (LT)0 && best < (LT)INFINITY);
-        if (bi != k) {
-          const int t = perm[k];
-          perm[k] = perm[bi];
-          perm[bi] = t;
+        __syncthreads();
+        LT best = s_key[buf][0];
+        int src = 0;
+#pragma unroll
+        for (int q = 1; q < kSrWarps; ++q)
+          if (s_key[buf][q] > best) {
+            best = s_key[buf][q];
+            src = q;
+          }
+        bad |= !(best > (LT)0 && best < (LT)INFINITY);
+        const int p = s_idx[buf][src];
+        if (tid == p) {
+          open = false;
+          s_piv[kk] = p;
+        }
+        if (open) {
+          const V l = sr_mul(v[kk], sr_recip(s_cand[buf][src][kk]));
+          v[kk] = l;
+#pragma unroll
+          for (int j = kk + 1; j < PB; ++j) sr_fnma(v[j], l, s_cand[buf][src][j]);
         }
       }
     }
+    if (own)
+#pragma unroll
+      for (int j = 0; j < PB; ++j)
+        if (j < nb) a[tid * n + c0 + j] = v[j];
     __syncthreads();
-    const int p = s_int[0];
-    bad |= s_int[1];
-    if (p != k)
-      for (int j = tid; j < n; j += kSrThreads) {
-        const V t = a[k * n + j];
-        a[k * n + j] = a[p * n + j];
-        a[p * n + j] = t;
+    // exchange row c0 + kk with the place where the step's pivot row is by then
+    {
+      int q[PB];
+#pragma unroll
+      for (int kk = 0; kk < PB; ++kk) {
+        q[kk] = kk < nb ? s_piv[kk] : c0 + kk;
+#pragma unroll
+        for (int m = 0; m < kk; ++m)
+          if (q[kk] == c0 + m) q[kk] = q[m];
       }
+#pragma unroll
+      for (int kk = 0; kk < PB; ++kk)
+        if (q[kk] != c0 + kk) {
+          if (tid < n) {
+            const V t = a[(c0 + kk) * n + tid];
+            a[(c0 + kk) * n + tid] = a[q[kk] * n + tid];
+            a[q[kk] * n + tid] = t;
+          }
+          if (tid == kSrThreads - 1) {
+            const int t = perm[c0 + kk];
+            perm[c0 + kk] = perm[q[kk]];
+            perm[q[kk]] = t;
+          }
+        }
+    }
     __syncthreads();
-    const V inv = sr_recip(a[k * n + k]);
-    for (int i = k + 1 + tid; i < n; i += kSrThreads) a[i * n + k] = sr_mul(a[i * n + k], inv);
-    __syncthreads();
-    // trailing update: rows over warps, columns over lanes
-    for (int i = k + 1 + warp; i < n; i += kSrWarps) {
-      const V lik = a[i * n + k];
-      for (int j = k + 1 + lane; j < n; j += 32) a[i * n + j] = sr_sub(a[i * n + j], sr_mul(lik, a[k * n + j]));
+    const int ct = n - c0 - PB;  // trailing columns
+    if (ct > 0) {
+      const int width = ct <= 32 ? 32 : (ct <= 64 ? 64 : kSrThreads);
+      const int col = tid % width, rg = tid / width, ng = kSrThreads / width;
+      const V* Lb = a + c0 * n + c0;  // the panel's unit lower triangle
+      V* at = a + c0 + PB + col;
+      V u[PB];
+#pragma unroll
+      for (int i = 0; i < PB; ++i) u[i] = col < ct ? at[(c0 + i) * n] : V{0, 0};
+#pragma unroll
+      for (int m = 0; m < PB; ++m)
+#pragma unroll
+        for (int i = m + 1; i < PB; ++i) sr_fnma(u[i], Lb[i * n + m], u[m]);
+      __syncthreads();  // every group has read the pivot rows
+      if (col < ct) {
+        if (rg == 0)
+#pragma unroll
+          for (int i = 0; i < PB; ++i) at[(c0 + i) * n] = u[i];
+        for (int i = c0 + PB + rg; i < n; i += ng) {
+          V w = at[i * n];
+#pragma unroll
+          for (int m = 0; m < PB; ++m) sr_fnma(w, a[i * n + c0 + m], u[m]);
+          at[i * n] = w;
+        }
+      }
     }
     __syncthreads();
   }
@@ -485,7 +577,6 @@ __global__ void __launch_bounds__(kSrThreads) sr_solve_kernel(SrArgs a) {
   double2* sv = reinterpret_cast<double2*>(sm_sr + o[6]);
   int* perm = reinterpret_cast<int*>(sm_sr + o[7]);
   double* red = reinterpret_cast<double*>(sm_sr + o[8]);
-  int* sint = reinterpret_cast<int*>(red + 32);
   const SrTables& tb = *a.tabs;
   const double2* S0f = a.S0 + (int64_t)f * n * n;
   const double2* Tf = a.T + (int64_t)f * n * n;
@@ -523,7 +614,7 @@ __global__ void __launch_bounds__(kSrThreads) sr_solve_kernel(SrArgs a) {
     }
   }
   __syncthreads();
-  const int singular = sr_factor<LT>(n, lu, perm, sint);
+  const int singular = sr_factor<LT>(n, lu, perm);
 
   // first solve
   for (int e = tid; e < nn1; e += kSrThreads) x[e] = sr_from<V>(rhs[perm[e / n1] * n1 + e % n1]);
