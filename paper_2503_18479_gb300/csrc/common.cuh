@@ -203,6 +203,32 @@ __host__ __device__ inline uint32_t swz128(uint32_t r, uint32_t kk) {
   return r * 128u + ((((kk >> 3) ^ (r & 7u)) & 7u) << 4) + ((kk & 7u) << 1);
 }
 
+// Whether the last of several K chunks of an operand holds the three pieces of its at most 16
+// columns side by side too (piece q at columns 16 q of piece 0's tile, where zeros would be): one
+// tile to copy instead of three. The tiles of the other pieces stay as they are for the kernels
+// that read chunk by chunk.
+__host__ __device__ inline bool tail_packed(int N, int npieces) {
+  const int t = N % kChunkK;
+  return npieces == 3 && N > kChunkK && t > 0 && t <= 16;
+}
+
+#ifdef __CUDACC__
+// piece q of row rr, column kg of a tensor-core operand with tiles of kTileN rows
+__device__ inline void put_piece(char* base, int64_t ntile, int64_t tile, int N, int npieces, uint32_t rr,
+                                 int kg, int q, __nv_bfloat16 h) {
+  static_assert(kTileN == kTileP, "tiles of both operands alike");
+  const int nkc = (N + kChunkK - 1) / kChunkK, kc = kg / kChunkK, kk = kg % kChunkK;
+  constexpr size_t tile_bytes = (size_t)kTileN * kChunkK * 2;
+  auto at = [&](int piece, int col) {
+    return reinterpret_cast<__nv_bfloat16*>(base + ((size_t)(piece * ntile + tile) * nkc + kc) * tile_bytes +
+                                            swz128(rr, col));
+  };
+  const bool packed = kc == nkc - 1 && tail_packed(N, npieces);
+  if (!packed || q > 0 || kk < 16 || kk >= 48) *at(q, kk) = h;
+  if (packed && q > 0 && kk < 16) *at(0, 16 * q + kk) = h;
+}
+#endif
+
 // Straight sides of the loops (basis.cu, write_sides), indexed by the loop's first vertex plus
 // the side's number, and what belongs to the loop as a whole.
 struct LoopInfo {

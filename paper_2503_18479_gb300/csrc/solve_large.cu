@@ -1005,9 +1005,7 @@ __global__ void __launch_bounds__(T, T == 128 ? 4 : (T == 256 ? 2 : 1)) solve_la
       const int nkc = (N + kChunkK - 1) / kChunkK;
       const int64_t ntile = (2 * a.n_cfg * F + kTileN - 1) / kTileN;
       char* base = reinterpret_cast<char*>(a.Bop + a.bop_off[si.s]);
-      const size_t tile_bytes = (size_t)kTileN * kChunkK * 2;
       for (int kg = tid; kg < nkc * kChunkK; kg += T) {
-        const int kc = kg / kChunkK, kk = kg % kChunkK;
         for (int c = 0; c < 2; ++c) {
           const int64_t n = 2 * (si.b * F + si.f) + c;
           const int64_t tile = n / kTileN;
@@ -1019,8 +1017,7 @@ __global__ void __launch_bounds__(T, T == 128 ? 4 : (T == 256 ? 2 : 1)) solve_la
             const __nv_bfloat16 h = __float2bfloat16_rn(rem);
             rem = rem - __bfloat162float(h);
             if (q == 0) rem += xl;
-            const size_t off = ((size_t)(q * ntile + tile) * nkc + kc) * tile_bytes + swz128(rr, kk);
-            *reinterpret_cast<__nv_bfloat16*>(base + off) = h;
+            put_piece(base, ntile, tile, N, a.npieces, rr, kg, q, h);
           }
         }
       }

@@ -786,10 +786,8 @@ solve_mixed_v4(SolveArgs a, int64_t n_sys) {
         const int nkc = (N + kChunkK - 1) / kChunkK;
         const int64_t ntile = (2 * a.n_cfg * F + kTileN - 1) / kTileN;
         char* base = reinterpret_cast<char*>(a.Bop + a.bop_off[si.s]);
-        const size_t tile_bytes = (size_t)kTileN * kChunkK * 2;
         for (int kg = r; kg < nkc * kChunkK; kg += NM) {
           const bool own = (kg == r) && real_row;
-          const int kc = kg / kChunkK, kc_k = kg % kChunkK;
 #pragma unroll
           for (int c = 0; c < 2; ++c) {
             const int64_t n = 2 * (si.b * F + si.f) + c;
@@ -804,8 +802,7 @@ solve_mixed_v4(SolveArgs a, int64_t n_sys) {
               const __nv_bfloat16 h = __float2bfloat16_rn(rem);
               rem = rem - __bfloat162float(h);
               if (q == 0) rem += xl;
-              size_t off = ((size_t)(q * ntile + tile) * nkc + kc) * tile_bytes + swz128(rr, kc_k);
-              *reinterpret_cast<__nv_bfloat16*>(base + off) = h;
+              put_piece(base, ntile, tile, N, a.npieces, rr, kg, q, h);
             }
           }
         }

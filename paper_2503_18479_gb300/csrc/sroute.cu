@@ -981,14 +981,13 @@ __global__ void sr_pack_kernel(int F, int64_t n_cfg_v, int Kv, int npieces, int6
                                const int64_t* __restrict__ bop_off, const double* __restrict__ I,
                                __nv_bfloat16* __restrict__ Bop) {
   const int s = blockIdx.y;
-  const int nkc = (Kv + kChunkK - 1) / kChunkK, Kpad = nkc * kChunkK;
+  const int Kpad = (Kv + kChunkK - 1) / kChunkK * kChunkK;
   const int64_t ntile = (2 * n_cfg_v + kTileN - 1) / kTileN;
-  const size_t tile_bytes = (size_t)kTileN * kChunkK * 2;
   char* base = reinterpret_cast<char*>(Bop + bop_off[s]);
   for (int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; idx < n_cfg_v * Kpad;
        idx += (int64_t)gridDim.x * blockDim.x) {
     const int64_t nsys = idx / Kpad;
-    const int kg = (int)(idx % Kpad), kc = kg / kChunkK, kk = kg % kChunkK;
+    const int kg = (int)(idx % Kpad);
     for (int c = 0; c < 2; ++c) {
       const int64_t row = 2 * nsys + c;
       const int64_t tile = row / kTileN;
@@ -1000,8 +999,7 @@ __global__ void sr_pack_kernel(int F, int64_t n_cfg_v, int Kv, int npieces, int6
         const __nv_bfloat16 h = __float2bfloat16_rn(rem);
         rem = rem - __bfloat162float(h);
         if (q == 0) rem += xl;
-        const size_t off = ((size_t)(q * ntile + tile) * nkc + kc) * tile_bytes + swz128(rr, kk);
-        *reinterpret_cast<__nv_bfloat16*>(base + off) = h;
+        put_piece(base, ntile, tile, Kv, npieces, rr, kg, q, h);
       }
     }
   }

@@ -106,6 +106,29 @@ struct RowWalk {
   }
 };
 
+// One point's 128 accumulator columns (64 systems, re and im) to the field
+__device__ __forceinline__ void store_tile(const SuperposeArgs& a, const Unit& x, int64_t sys0, int64_t fpo,
+                                           int64_t nsys, int64_t p, const float* v) {
+  if (p >= x.P) return;
+  RowWalk w(a, x, sys0, fpo, p);
+  if (w.even && sys0 + kTileN / 2 <= nsys) {
+    float2* dst = w.dst;
+    const int64_t stride = w.stride;
+#pragma unroll
+    for (int i = 0; i < kTileN / 2; ++i) {
+      st_cs_f2(dst, v[2 * i], v[2 * i + 1]);
+      dst += stride;
+    }
+  } else {
+    const int n = (int)min((int64_t)kTileN / 2, nsys - sys0);
+#pragma unroll
+    for (int i = 0; i < kTileN / 2; ++i) {
+      if (i < n) st_cs_f2(w.dst, v[2 * i], v[2 * i + 1]);
+      w.next();
+    }
+  }
+}
+
 template <int NPIECE>
 __global__ void __launch_bounds__(kThreads, 1) superpose_tc_kernel(SuperposeArgs a, int32_t* err) {
   constexpr int NSTAGE = NPIECE == 3 ? 2 : 4;
@@ -361,25 +384,7 @@ __global__ void __launch_bounds__(kThreads, 1) superpose_tc_kernel(SuperposeArgs
         acc = 0;
         aphase ^= 1u;
       }
-      if (p < x.P) {
-        RowWalk w(a, x, sys0, fpo, p);
-        if (w.even && sys0 + kTileN / 2 <= nsys) {
-          float2* dst = w.dst;
-          const int64_t stride = w.stride;
-#pragma unroll
-          for (int i = 0; i < kTileN / 2; ++i) {
-            st_cs_f2(dst, v[2 * i], v[2 * i + 1]);
-            dst += stride;
-          }
-        } else {
-          const int n = (int)min((int64_t)kTileN / 2, nsys - sys0);
-#pragma unroll
-          for (int i = 0; i < kTileN / 2; ++i) {
-            if (i < n) st_cs_f2(w.dst, v[2 * i], v[2 * i + 1]);
-            w.next();
-          }
-        }
-      }
+      store_tile(a, x, sys0, fpo, nsys, p, v);
     }
   }
 
@@ -393,10 +398,280 @@ __global__ void __launch_bounds__(kThreads, 1) superpose_tc_kernel(SuperposeArgs
   }
 }
 
+// One structure whose column tile (NPIECE pieces of every K chunk) fits in shared memory beside a
+// ring for the point tiles: the column tile stays while the point tiles pass, piece by piece. With
+// both operands through stages of a chunk, a unit of more than one chunk read both tiles again
+// each time (65,600 points, 8192 columns, K = 130: 288 KB a unit, 970 us; resident 913 us), and a
+// last chunk of at most 16 columns took three tiles for six MMAs; as one tile with its pieces side
+// by side (tail_packed): 783 us. With one chunk the stages keep their column tile anyway and
+// hold more of the point tiles (64 ports: 381 us in both forms), so that form stays there.
+// Barriers: full/empty per ring slot, bfull/bempty per chunk of a column tile; bempty is
+// committed by the last unit that reads it.
+constexpr int kSlots = 14;       // 16 KB each: the column tile first, the ring behind it
+constexpr int kResidentMax = 9;  // of them at most for the column tile
+
+// An MMA of M = 128 takes much the same time for N = 128 and N = 256, so the products of an A
+// piece with the first two B pieces go out as one MMA of N = 256: the pieces' tiles follow each
+// other in shared memory as the rows of one operand, and the second one's products have an
+// accumulator of their own, which the epilogue adds (783 -> 648 us for the 65,600 points below).
+// The A pieces come in the order 1, 2, 0, because the first of them starts both accumulators.
+constexpr uint32_t kIdesc256 = (kIdesc & ~(0x3fu << 17)) | ((256u >> 3) << 17);
+
+__device__ __forceinline__ constexpr int a_piece(int npieces, int t) {
+  return npieces == 3 ? (t == 0 ? 1 : (t == 1 ? 2 : 0)) : 0;
+}
+
+// 16 KB tiles that one side of a unit takes
+__host__ __device__ inline int unit_tiles(int N, int nkc, int npieces) {
+  return tail_packed(N, npieces) ? (nkc - 1) * npieces + 1 : nkc * npieces;
+}
+
+template <int NPIECE>
+__global__ void __launch_bounds__(kThreads, 1) superpose_tc_resident_kernel(SuperposeArgs a, int32_t* err) {
+  constexpr uint32_t kAcc = NPIECE == 3 ? 256 : 128;  // TMEM columns of an accumulator
+  extern __shared__ __align__(1024) unsigned char smem_dyn[];
+  const uintptr_t sbase = (reinterpret_cast<uintptr_t>(smem_dyn) + 1023) & ~uintptr_t(1023);
+  unsigned char* sB = reinterpret_cast<unsigned char*>(sbase);
+  uint64_t* full = reinterpret_cast<uint64_t*>(sB + kSlots * kTileBytes);  // [kSlots]
+  uint64_t* empty = full + kSlots;                                         // [kSlots]
+  uint64_t* bfull = empty + kSlots;                                        // [kResidentMax]
+  uint64_t* bempty = bfull + kResidentMax;                                 // [kResidentMax]
+  uint64_t* tfull = bempty + kResidentMax;                                 // [2]
+  uint64_t* tempty = tfull + 2;                                            // [2]
+  uint64_t* mdone = tempty + 2;
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(mdone + 1);
+
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int nkc = a.uni.nkc, N = a.uni.N;
+  const bool packed = tail_packed(N, NPIECE);
+  const int nB = unit_tiles(N, nkc, NPIECE), ring = kSlots - nB;
+  unsigned char* sA = sB + nB * kTileBytes;
+  const int64_t nptile = a.uni.nptile, nntile = a.uni.nntile;
+  const int64_t u_begin = a.total_units * blockIdx.x / gridDim.x;
+  const int64_t u_end = a.total_units * (blockIdx.x + 1) / gridDim.x;
+
+  if (threadIdx.x == 0) {
+    for (int i = 0; i < 2 * (kSlots + kResidentMax); ++i) mbar_init(&full[i], 1);
+    for (int i = 0; i < 2; ++i) {
+      mbar_init(&tfull[i], 1);
+      mbar_init(&tempty[i], 128);
+    }
+    mbar_init(mdone, 1);
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
+  if (warp == 1) {
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(
+                     smem_u32(tmem_slot)),
+                 "r"(2 * kAcc)
+                 : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+  }
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  const uint32_t tmem_base = *tmem_slot;
+
+  if (warp == 0) {
+    // ---------------- producer ----------------
+    if (lane == 0) {
+      const unsigned char* Ab = reinterpret_cast<const unsigned char*>(a.Aop);
+      const unsigned char* Bb = reinterpret_cast<const unsigned char*>(a.Bop);
+      int slot = 0, nb = 0;  // ring slot, column tiles begun
+      uint32_t phase = 0;
+      int64_t copies = 0, held = -1;
+      int b_chunks = 0;  // chunks of the current column tile asked for
+      bool ok = true;
+      for (int64_t u = u_begin; u < u_end && ok; ++u) {
+        const int64_t nt = u / nptile, pt = u - nt * nptile;
+        const bool fresh = nt != held;
+        if (fresh) {
+          held = nt;
+          ++nb;
+          b_chunks = 0;
+        }
+        for (int kc = 0; kc < nkc && ok; ++kc) {
+          const int np = packed && kc == nkc - 1 ? 1 : NPIECE;
+          if (fresh) {
+            ok = mbar_wait(&bempty[kc], (uint32_t)nb & 1u, err, 1);
+            if (!ok) break;
+            mbar_arrive_expect_tx(&bfull[kc], np * kTileBytes);
+            for (int q = 0; q < np; ++q)
+              bulk_g2s(sB + (kc * NPIECE + q) * kTileBytes,
+                       Bb + ((size_t)(q * nntile + nt) * nkc + kc) * kTileBytes, kTileBytes, &bfull[kc]);
+            b_chunks = kc + 1;
+          }
+          for (int i = 0; i < np; ++i) {
+            const int q = np == 1 ? 0 : a_piece(NPIECE, i);
+            ok = mbar_wait(&empty[slot], phase ^ 1u, err, 1);
+            if (!ok) break;
+            mbar_arrive_expect_tx(&full[slot], kTileBytes);
+            bulk_g2s(sA + slot * kTileBytes, Ab + ((size_t)(q * nptile + pt) * nkc + kc) * kTileBytes,
+                     kTileBytes, &full[slot]);
+            ++copies;
+            if (++slot == ring) {
+              slot = 0;
+              phase ^= 1u;
+            }
+          }
+        }
+      }
+      // no copy may still be in flight when the CTA exits: the last use of every slot and chunk
+      for (int i = 0; i < ring && i < copies; ++i)
+        mbar_wait(&full[i], (uint32_t)(((copies - 1 - i) / ring) & 1), err, 5);
+      for (int kc = 0; kc < nkc; ++kc) {
+        const int uses = kc < b_chunks ? nb : nb - 1;
+        if (uses > 0) mbar_wait(&bfull[kc], (uint32_t)(uses - 1) & 1u, err, 5);
+      }
+    }
+  } else if (warp == 1) {
+    // ---------------- MMA issuer ----------------
+    if (lane == 0) {
+      int slot = 0, nb = 0, acc = 0;
+      uint32_t phase = 0, aphase = 0;
+      int64_t held = -1;
+      bool ok = true;
+      for (int64_t u = u_begin; u < u_end && ok; ++u) {
+        const int64_t nt = u / nptile;
+        const bool fresh = nt != held, last = u + 1 == u_end || (u + 1) / nptile != nt;
+        if (fresh) {
+          held = nt;
+          ++nb;
+        }
+        ok = mbar_wait(&tempty[acc], aphase ^ 1u, err, 2);
+        if (!ok) break;
+        tc_fence_after();
+        const uint32_t d_tmem = tmem_base + (uint32_t)acc * kAcc;
+        for (int kc = 0; kc < nkc && ok; ++kc) {
+          if (fresh) {
+            ok = mbar_wait(&bfull[kc], (uint32_t)(nb - 1) & 1u, err, 3);
+            if (!ok) break;
+          }
+          const int ksteps = min(kChunkK / 16, (N - kc * kChunkK + 15) / 16);
+          const uint32_t b0 = smem_u32(sB) + (uint32_t)(kc * NPIECE) * kTileBytes;
+          if (packed && kc == nkc - 1) {  // piece q is K step q of the one tile
+            ok = mbar_wait(&full[slot], phase, err, 3);
+            if (!ok) break;
+            tc_fence_after();
+            const uint64_t da = make_desc(smem_u32(sA) + (uint32_t)slot * kTileBytes), db = make_desc(b0);
+#pragma unroll
+            for (int qa = NPIECE - 1; qa >= 0; --qa)
+#pragma unroll
+              for (int qb = NPIECE - 1 - qa; qb >= 0; --qb)
+                mma_bf16(d_tmem, da + (uint64_t)(qa * 2), db + (uint64_t)(qb * 2),
+                         1u);
+            mma_commit(&empty[slot]);
+            if (++slot == ring) {
+              slot = 0;
+              phase ^= 1u;
+            }
+            if (last) mma_commit(&bempty[kc]);
+            continue;
+          }
+          // piece pairs of order >= 2^-16
+#pragma unroll
+          for (int i = 0; i < NPIECE; ++i) {
+            const int qa = a_piece(NPIECE, i);
+            ok = mbar_wait(&full[slot], phase, err, 3);
+            if (!ok) break;
+            tc_fence_after();
+            const uint64_t da = make_desc(smem_u32(sA) + (uint32_t)slot * kTileBytes);
+            auto steps = [&](int qb, uint32_t idesc) {
+              const uint64_t db = make_desc(b0 + qb * kTileBytes);
+#pragma unroll
+              for (int kk = 0; kk < kChunkK / 16; ++kk)
+                if (kk < ksteps)
+                  mma_bf16(d_tmem, da + (uint64_t)(kk * 2), db + (uint64_t)(kk * 2),
+                           (kc > 0 || i > 0 || kk > 0) ? 1u : 0u, idesc);
+            };
+            if constexpr (NPIECE == 3) {
+              if (qa == 0) steps(2, kIdesc);
+              steps(0, qa == 2 ? kIdesc : kIdesc256);
+            } else {
+              steps(0, kIdesc);
+            }
+            mma_commit(&empty[slot]);
+            if (++slot == ring) {
+              slot = 0;
+              phase ^= 1u;
+            }
+          }
+          if (ok && last) mma_commit(&bempty[kc]);
+        }
+        if (!ok) break;
+        mma_commit(&tfull[acc]);
+        if (++acc == 2) {
+          acc = 0;
+          aphase ^= 1u;
+        }
+      }
+      // every MMA issued by this thread has finished before TMEM is released
+      mma_commit(mdone);
+      mbar_wait(mdone, 0, err, 6);
+    }
+  } else {
+    // ---------------- epilogue (warps 2..5) ----------------
+    const int quarter = warp & 3;  // TMEM lanes 32*quarter .. +31
+    int acc = 0;
+    uint32_t aphase = 0;
+    for (int64_t u = u_begin; u < u_end; ++u) {
+      const Unit x = unit_info(a, u);
+      int ok = (lane == 0) ? (int)mbar_wait(&tfull[acc], aphase, err, 4) : 1;
+      ok = __shfl_sync(0xffffffffu, ok, 0);
+      if (!ok) break;
+      mbar_wait(&tfull[acc], aphase, err, 4);  // already complete: acquire for every lane
+      tc_fence_after();
+      float v[128];
+      const uint32_t taddr = tmem_base + ((uint32_t)(quarter * 32) << 16) + (uint32_t)acc * kAcc;
+#pragma unroll
+      for (int c = 0; c < 4; ++c) tmem_ld32(taddr + c * 32, v + c * 32);
+      tmem_wait_ld();
+      if constexpr (NPIECE == 3) {
+#pragma unroll
+        for (int c = 0; c < 4; ++c) {
+          float y[32];
+          tmem_ld32(taddr + 128 + c * 32, y);
+          tmem_wait_ld();
+#pragma unroll
+          for (int i = 0; i < 32; ++i) v[32 * c + i] += y[i];
+        }
+      }
+      tc_fence_before();
+      mbar_arrive(&tempty[acc]);
+      if (++acc == 2) {
+        acc = 0;
+        aphase ^= 1u;
+      }
+      store_tile(a, x, x.nt * (kTileN / 2), 0, a.n_cfg * x.F, x.pt * kTileP + quarter * 32 + lane, v);
+    }
+  }
+
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  if (warp == 1) {
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base),
+                 "r"(2 * kAcc)
+                 : "memory");
+  }
+}
+
 template <int NPIECE>
 size_t smem_bytes() {
   constexpr int NSTAGE = NPIECE == 3 ? 2 : 4;
   return 1024 + (size_t)NSTAGE * 2 * NPIECE * kTileBytes + 8 * (2 * NSTAGE + 5) + 16;
+}
+
+constexpr size_t kResidentSmem = 1024 + (size_t)kSlots * kTileBytes + 8 * (2 * (kSlots + kResidentMax) + 5) + 16;
+
+template <int NPIECE>
+cudaError_t launch(const SuperposeArgs& a, int64_t grid, int32_t* err, cudaStream_t st) {
+  const bool resident = a.uni.on && a.uni.nkc > 1 && unit_tiles(a.uni.N, a.uni.nkc, NPIECE) <= kResidentMax;
+  const auto kernel = resident ? superpose_tc_resident_kernel<NPIECE> : superpose_tc_kernel<NPIECE>;
+  const size_t sm = resident ? kResidentSmem : smem_bytes<NPIECE>();
+  const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+  if (e != cudaSuccess) return e;
+  kernel<<<(unsigned)grid, kThreads, sm, st>>>(a, err);
+  return cudaSuccess;
 }
 
 }  // namespace tc
@@ -413,19 +688,8 @@ cudaError_t launch_superpose_tc(const SuperposeArgs& a, mts_precision prec, cuda
   int64_t grid = a.total_units < g_num_sms ? a.total_units : g_num_sms;
   int32_t* err = a.err;
   if (err == nullptr) return cudaErrorInvalidValue;
-  if (prec == MTS_MIXED) {
-    size_t sm = tc::smem_bytes<3>();
-    cudaError_t e = cudaFuncSetAttribute(tc::superpose_tc_kernel<3>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-    if (e != cudaSuccess) return e;
-    tc::superpose_tc_kernel<3><<<(unsigned)grid, tc::kThreads, sm, st>>>(a, err);
-  } else {
-    size_t sm = tc::smem_bytes<1>();
-    cudaError_t e = cudaFuncSetAttribute(tc::superpose_tc_kernel<1>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-    if (e != cudaSuccess) return e;
-    tc::superpose_tc_kernel<1><<<(unsigned)grid, tc::kThreads, sm, st>>>(a, err);
-  }
+  const cudaError_t e = prec == MTS_MIXED ? tc::launch<3>(a, grid, err, st) : tc::launch<1>(a, grid, err, st);
+  if (e != cudaSuccess) return e;
   note_launch();
   return cudaGetLastError();
 }
