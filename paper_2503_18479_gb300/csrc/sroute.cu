@@ -177,28 +177,90 @@ __device__ inline void sr_split(double2 v, float2& h, float2& l) {
   l = make_float2((float)(v.x - (double)h.x), (float)(v.y - (double)h.y));
 }
 
-// sum_j M_j x_j (conj(M_j) x_j when CONJ) for complex M = Mh + Ml (element j at j*ms) and
-// x = xh + xl (element j at j*xs): the hi x hi products exactly, the cross terms in FP32,
-// all accumulated in double-float (about 2^-44 relative).
+// Row dot products, eight lanes a row. A thread per row left half of the CTA idle and waited on
+// one batch of L2 loads after another (the matrices do not fit in what shared memory leaves of
+// L1): these sums were a third of the solve's and more than half of the adjoint's time. Eight
+// lanes read a row in 64- or 128-byte pieces, all of a lane's up to twelve entries in flight.
+constexpr int kSrLaneEntries = kSrMaxN0 / 8;
+
+__device__ __forceinline__ void sr_df_add(float& hi, float& lo, float h, float l) {
+  const float s = __fadd_rn(hi, h), bb = __fsub_rn(s, hi);
+  lo = __fadd_rn(__fadd_rn(lo, l), __fadd_rn(__fsub_rn(hi, __fsub_rn(s, bb)), __fsub_rn(h, bb)));
+  hi = s;
+}
+
+// sum_j M_j x_j (conj(M_j) x_j when CONJ) for complex M_j = (hi, lo) quadruples and x = xh + xl
+// (element j at j*xs, shared memory): the hi x hi products exactly, the cross terms in FP32, all
+// accumulated in double-float (about 2^-44 relative). Result in all eight lanes.
 template <bool CONJ>
-__device__ double2 sr_df_dot(const float2* __restrict__ Mh, const float2* __restrict__ Ml,
-                             int ms, const float2* xh, const float2* xl, int xs, int n) {
+__device__ double2 sr_df_dot(const float4* __restrict__ M, const float2* xh, const float2* xl, int xs, int n) {
+  const int sub = threadIdx.x & 7;
+  float4 m[kSrLaneEntries];
+#pragma unroll
+  for (int t = 0; t < kSrLaneEntries; ++t) {
+    const int j = sub + 8 * t;
+    m[t] = j < n ? M[j] : make_float4(0.f, 0.f, 0.f, 0.f);
+  }
   float rh = 0.f, rl = 0.f, ih = 0.f, il = 0.f;
-  for (int j = 0; j < n; ++j) {
-    float2 a = Mh[(int64_t)j * ms], c = Ml[(int64_t)j * ms];
-    if (CONJ) {
-      a.y = -a.y;
-      c.y = -c.y;
+#pragma unroll
+  for (int t = 0; t < kSrLaneEntries; ++t) {
+    const int j = sub + 8 * t;
+    if (j < n) {
+      const float ax = m[t].x, ay = CONJ ? -m[t].y : m[t].y, cx = m[t].z, cy = CONJ ? -m[t].w : m[t].w;
+      const float2 p = xh[j * xs], q = xl[j * xs];
+      sr_df_acc(rh, rl, ax, p.x);
+      sr_df_acc(rh, rl, -ay, p.y);
+      sr_df_acc(ih, il, ax, p.y);
+      sr_df_acc(ih, il, ay, p.x);
+      rl = fmaf(ax, q.x, fmaf(-ay, q.y, fmaf(cx, p.x, fmaf(-cy, p.y, rl))));
+      il = fmaf(ax, q.y, fmaf(ay, q.x, fmaf(cx, p.y, fmaf(cy, p.x, il))));
     }
-    const float2 p = xh[j * xs], q = xl[j * xs];
-    sr_df_acc(rh, rl, a.x, p.x);
-    sr_df_acc(rh, rl, -a.y, p.y);
-    sr_df_acc(ih, il, a.x, p.y);
-    sr_df_acc(ih, il, a.y, p.x);
-    rl = fmaf(a.x, q.x, fmaf(-a.y, q.y, fmaf(c.x, p.x, fmaf(-c.y, p.y, rl))));
-    il = fmaf(a.x, q.y, fmaf(a.y, q.x, fmaf(c.x, p.y, fmaf(c.y, p.x, il))));
+  }
+  __syncwarp();
+#pragma unroll
+  for (int o = 4; o > 0; o >>= 1) {
+    const float rh2 = __shfl_xor_sync(0xffffffffu, rh, o), rl2 = __shfl_xor_sync(0xffffffffu, rl, o);
+    const float ih2 = __shfl_xor_sync(0xffffffffu, ih, o), il2 = __shfl_xor_sync(0xffffffffu, il, o);
+    sr_df_add(rh, rl, rh2, rl2);
+    sr_df_add(ih, il, ih2, il2);
   }
   return make_double2((double)rh + (double)rl, (double)ih + (double)il);
+}
+
+// the same with FP32 entries, products and sums; at most kSrMaxN0 entries
+template <bool CONJ, typename X>
+__device__ float2 sr_f32_dot(const float2* __restrict__ M, X x, int n) {
+  const int sub = threadIdx.x & 7;
+  float2 m[kSrLaneEntries];
+#pragma unroll
+  for (int t = 0; t < kSrLaneEntries; ++t) {
+    const int j = sub + 8 * t;
+    m[t] = j < n ? M[j] : make_float2(0.f, 0.f);
+  }
+  float2 v = make_float2(0.f, 0.f);
+#pragma unroll
+  for (int t = 0; t < kSrLaneEntries; ++t) {
+    const int j = sub + 8 * t;
+    if (j < n) v = sr_add(v, sr_mul(CONJ ? sr_conj(m[t]) : m[t], x(j)));
+  }
+  __syncwarp();
+#pragma unroll
+  for (int o = 4; o > 0; o >>= 1) {
+    v.x += __shfl_xor_sync(0xffffffffu, v.x, o);
+    v.y += __shfl_xor_sync(0xffffffffu, v.y, o);
+  }
+  return v;
+}
+
+// f(e) for e < count by the CTA's groups of eight lanes, put(e, value) by the first of them
+template <typename F, typename Put>
+__device__ __forceinline__ void sr_rows(int count, F f, Put put) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  for (int e0 = 4 * warp; e0 < count; e0 += 4 * kSrWarps) {
+    const int e = e0 + (lane >> 3);
+    const auto v = f(min(e, count - 1));  // every lane takes part in the shuffles
+    if (e < count && (lane & 7) == 0) put(e, v);
+  }
 }
 
 // c -= a b (complex)
@@ -361,7 +423,9 @@ __device__ int sr_factor(int n, typename SrT<LT>::V* a, int* perm) {
 // Triangular sweeps with the factors of sr_factor, one warp per right-hand-side column (n1
 // columns, warps take columns w, w + 4, ...): lane l holds the unknowns of rows l, l + 32,
 // l + 64 in registers; the unknown of step k is broadcast from its lane by a shuffle, so a
-// sweep needs no CTA barrier (one at the end publishes x).
+// sweep needs no CTA barrier (one at the end publishes x). The bound is the chain from one
+// unknown to the next: the next step's entries are loaded ahead, the inverse diagonal is formed
+// once by all lanes, and the slot of step k is known at compile time.
 template <typename V>
 __device__ inline V sr_bcast(V v, int src) {
   V r;
@@ -370,8 +434,57 @@ __device__ inline V sr_bcast(V v, int src) {
   return r;
 }
 
+// One sweep over the unknowns v (three slots of 32 rows): rows after k (FWD) or before k take
+// step k's unknown, divided by the diagonal first where DIAG. Entry (i, k) of the triangle is
+// a[i][k], or conj(a[k][i]) where H.
+template <bool H, bool DIAG, bool FWD, typename V>
+__device__ __forceinline__ void sr_sweep(int n, const V* a, V* v) {
+  const int lane = threadIdx.x & 31;
+  auto at = [&](int i, int k) -> V { return H ? sr_conj(a[k * n + i]) : a[i * n + k]; };
+  V d[3];
+  if constexpr (DIAG) {
+#pragma unroll
+    for (int s = 0; s < 3; ++s) {
+      const int i = lane + 32 * s;
+      d[s] = i < n ? sr_recip(at(i, i)) : V{0, 0};
+    }
+  }
+#pragma unroll
+  for (int b = 0; b < 3; ++b) {
+    const int ks = FWD ? b : 2 - b;
+    const int k0 = 32 * ks, steps = min(n - k0, 32);
+    auto live = [&](int s, int k) {
+      const int i = lane + 32 * s;
+      return FWD ? (s >= ks && i > k && i < n) : (s <= ks && i < k);
+    };
+    auto load = [&](int k, V* e) {
+#pragma unroll
+      for (int s = 0; s < 3; ++s)
+        if (FWD ? s >= ks : s <= ks) e[s] = live(s, k) ? at(lane + 32 * s, k) : V{0, 0};
+    };
+    V e[3];
+    if (steps > 0) load(FWD ? k0 : k0 + steps - 1, e);
+    for (int q = 0; q < steps; ++q) {
+      const int k = FWD ? k0 + q : k0 + steps - 1 - q;
+      V next[3] = {};
+      if (q + 1 < steps) load(FWD ? k + 1 : k - 1, next);
+      V x = v[ks];
+      if constexpr (DIAG) x = sr_mul(x, d[ks]);
+      x = sr_bcast(x, k & 31);
+      if (DIAG && lane == (k & 31)) v[ks] = x;
+#pragma unroll
+      for (int s = 0; s < 3; ++s)
+        if (live(s, k)) sr_fnma(v[s], e[s], x);
+#pragma unroll
+      for (int s = 0; s < 3; ++s) e[s] = next[s];
+    }
+  }
+}
+
 // x <- U^-1 L^-1 x for the n1 columns of x ([n][n1]; x already row-permuted by P), n <= 96.
-template <typename V>
+// H: x <- (L^H)^-1 (U^H)^-1 x. With P A = L U, A^H = U^H L^H P, so A^H z = g is
+// z = P^T (L^H)^-1 (U^H)^-1 g; the caller applies P^T (z[perm[i]] = x[i]).
+template <bool H, typename V>
 __device__ void sr_solve_lu(int n, int n1, const V* a, V* x) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   for (int c = warp; c < n1; c += kSrWarps) {
@@ -381,79 +494,8 @@ __device__ void sr_solve_lu(int n, int n1, const V* a, V* x) {
       const int i = lane + 32 * s;
       v[s] = i < n ? x[i * n1 + c] : V{0, 0};
     }
-    for (int k = 0; k + 1 < n; ++k) {  // L y = P b (unit diagonal)
-      const int ks = k >> 5;
-      const V mine = ks == 0 ? v[0] : (ks == 1 ? v[1] : v[2]);
-      const V xk = sr_bcast(mine, k & 31);
-#pragma unroll
-      for (int s = 0; s < 3; ++s) {
-        const int i = lane + 32 * s;
-        if (i > k && i < n) v[s] = sr_sub(v[s], sr_mul(a[i * n + k], xk));
-      }
-    }
-    for (int k = n - 1; k >= 0; --k) {  // U x = y
-      const int ks = k >> 5;
-      if (lane == (k & 31)) {
-        const V d = sr_recip(a[k * n + k]);
-        if (ks == 0) v[0] = sr_mul(v[0], d);
-        else if (ks == 1) v[1] = sr_mul(v[1], d);
-        else v[2] = sr_mul(v[2], d);
-      }
-      const V mine = ks == 0 ? v[0] : (ks == 1 ? v[1] : v[2]);
-      const V xk = sr_bcast(mine, k & 31);
-#pragma unroll
-      for (int s = 0; s < 3; ++s) {
-        const int i = lane + 32 * s;
-        if (i < k) v[s] = sr_sub(v[s], sr_mul(a[i * n + k], xk));
-      }
-    }
-#pragma unroll
-    for (int s = 0; s < 3; ++s) {
-      const int i = lane + 32 * s;
-      if (i < n) x[i * n1 + c] = v[s];
-    }
-  }
-  __syncthreads();
-}
-
-// With P A = L U, A^H = U^H L^H P, so A^H z = g is z = P^T (L^H)^-1 (U^H)^-1 g; this applies
-// (L^H)^-1 (U^H)^-1 and the caller applies P^T (z[perm[i]] = x[i]).
-template <typename V>
-__device__ void sr_solve_lu_h(int n, int n1, const V* a, V* x) {
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  for (int c = warp; c < n1; c += kSrWarps) {
-    V v[3];
-#pragma unroll
-    for (int s = 0; s < 3; ++s) {
-      const int i = lane + 32 * s;
-      v[s] = i < n ? x[i * n1 + c] : V{0, 0};
-    }
-    for (int k = 0; k < n; ++k) {  // U^H t = g: row i of U^H is conj(column i of U)
-      const int ks = k >> 5;
-      if (lane == (k & 31)) {
-        const V d = sr_recip(sr_conj(a[k * n + k]));
-        if (ks == 0) v[0] = sr_mul(v[0], d);
-        else if (ks == 1) v[1] = sr_mul(v[1], d);
-        else v[2] = sr_mul(v[2], d);
-      }
-      const V mine = ks == 0 ? v[0] : (ks == 1 ? v[1] : v[2]);
-      const V xk = sr_bcast(mine, k & 31);
-#pragma unroll
-      for (int s = 0; s < 3; ++s) {
-        const int i = lane + 32 * s;
-        if (i > k && i < n) v[s] = sr_sub(v[s], sr_mul(sr_conj(a[k * n + i]), xk));
-      }
-    }
-    for (int k = n - 1; k > 0; --k) {  // L^H s = t (unit diagonal)
-      const int ks = k >> 5;
-      const V mine = ks == 0 ? v[0] : (ks == 1 ? v[1] : v[2]);
-      const V xk = sr_bcast(mine, k & 31);
-#pragma unroll
-      for (int s = 0; s < 3; ++s) {
-        const int i = lane + 32 * s;
-        if (i < k) v[s] = sr_sub(v[s], sr_mul(sr_conj(a[k * n + i]), xk));
-      }
-    }
+    sr_sweep<H, H, true>(n, a, v);    // L (unit diagonal), or U^H
+    sr_sweep<H, !H, false>(n, a, v);  // U, or L^H (unit diagonal)
 #pragma unroll
     for (int s = 0; s < 3; ++s) {
       const int i = lane + 32 * s;
@@ -515,8 +557,10 @@ struct SrArgs {
   const double* loss_weight;   // [F][n1][L] or nullptr
   const double2* loss_offset;  // [F][n1][L] or nullptr
   const SrTables* tabs;
-  // FP32 factors only: S0 and T as hi/lo float pairs, loss-point rows of the field in FP32
-  const float2 *S0h, *S0l, *Th, *Tl, *fl32;
+  // FP32 factors only: S0 and T in FP32, as (hi, lo) quadruples, and those transposed; loss-point
+  // rows of the field in FP32, and transposed
+  const float2 *S0h, *Th, *fl32, *flT;
+  const float4 *S0q, *Tq, *S0t, *Tt;
   double2* W;        // tape [n_cfg F][n0][n1]
   double2* W_out;    // optional copy
   void* lu;          // tape [n_cfg F][n0][n0] (float2 or double2)
@@ -594,24 +638,65 @@ __global__ void __launch_bounds__(kSrThreads) sr_solve_kernel(SrArgs a) {
   }
   // A = 1 - S_C,const11 S0 - sum over S11 entries v e_r S0[c, :]
   const int lane = tid & 31, warp = tid >> 5;
-  for (int i = warp; i < n; i += kSrWarps)
-  for (int j = lane; j < n; j += 32) {
-    const int e = i * n + j;
-    if constexpr (kDF) {  // the factors are FP32: assemble A in FP32
-      float2 v = make_float2(i == j ? 1.f : 0.f, 0.f);
-      if (tnz) v = sr_sub(v, a.Th[fo + e]);
-      for (int q = tb.r_ptr[i]; q < tb.r_ptr[i + 1]; ++q) {
-        const double2 s = sv[tb.r_var[q]];
-        v = sr_sub(v, sr_mul(make_float2((float)s.x, (float)s.y), a.S0h[fo + tb.r_col[q] * n + j]));
+  if constexpr (kDF) {
+    // the factors are FP32: A in FP32, four rows of a warp together, so that the table entries of
+    // all and then the first S0 rows of all are in flight at once
+    constexpr int RB = 4, JB = kSrMaxN0 / 32;
+    for (int i0 = warp; i0 < n; i0 += RB * kSrWarps) {
+      int q0[RB], q1[RB], col[RB];
+      float2 sf[RB], s0[RB][JB];
+#pragma unroll
+      for (int u = 0; u < RB; ++u) {
+        const int i = i0 + u * kSrWarps;
+        q0[u] = i < n ? tb.r_ptr[i] : 0;
+        q1[u] = i < n ? tb.r_ptr[i + 1] : 0;
       }
-      lu[e] = sr_from<V>(make_double2(v.x, v.y));
-    } else {
-      double2 v = make_double2(i == j ? 1.0 : 0.0, 0.0);
-      if (tnz) v = sr_sub(v, Tf[e]);
-      for (int q = tb.r_ptr[i]; q < tb.r_ptr[i + 1]; ++q)
-        v = sr_sub(v, sr_mul(sv[tb.r_var[q]], S0f[tb.r_col[q] * n + j]));
-      lu[e] = sr_from<V>(v);
+#pragma unroll
+      for (int u = 0; u < RB; ++u) {
+        col[u] = 0;
+        sf[u] = make_float2(0.f, 0.f);
+        if (q0[u] < q1[u]) {
+          const double2 v = sv[tb.r_var[q0[u]]];
+          sf[u] = make_float2((float)v.x, (float)v.y);
+          col[u] = tb.r_col[q0[u]];
+        }
+      }
+#pragma unroll
+      for (int u = 0; u < RB; ++u)
+#pragma unroll
+        for (int t = 0; t < JB; ++t) {
+          const int j = lane + 32 * t;
+          s0[u][t] = q0[u] < q1[u] && j < n ? a.S0h[fo + col[u] * n + j] : make_float2(0.f, 0.f);
+        }
+#pragma unroll
+      for (int u = 0; u < RB; ++u) {
+        const int i = i0 + u * kSrWarps;
+#pragma unroll
+        for (int t = 0; t < JB; ++t) {
+          const int j = lane + 32 * t;
+          if (i < n && j < n) {
+            float2 v = make_float2(i == j ? 1.f : 0.f, 0.f);
+            if (tnz) v = sr_sub(v, a.Th[fo + i * n + j]);
+            if (q0[u] < q1[u]) v = sr_sub(v, sr_mul(sf[u], s0[u][t]));
+            for (int q = q0[u] + 1; q < q1[u]; ++q) {
+              const double2 s = sv[tb.r_var[q]];
+              v = sr_sub(v, sr_mul(make_float2((float)s.x, (float)s.y), a.S0h[fo + tb.r_col[q] * n + j]));
+            }
+            lu[i * n + j] = sr_from<V>(make_double2(v.x, v.y));
+          }
+        }
+      }
     }
+  } else {
+    for (int i = warp; i < n; i += kSrWarps)
+      for (int j = lane; j < n; j += 32) {
+        const int e = i * n + j;
+        double2 v = make_double2(i == j ? 1.0 : 0.0, 0.0);
+        if (tnz) v = sr_sub(v, Tf[e]);
+        for (int q = tb.r_ptr[i]; q < tb.r_ptr[i + 1]; ++q)
+          v = sr_sub(v, sr_mul(sv[tb.r_var[q]], S0f[tb.r_col[q] * n + j]));
+        lu[e] = sr_from<V>(v);
+      }
   }
   __syncthreads();
   const int singular = sr_factor<LT>(n, lu, perm);
@@ -619,7 +704,7 @@ __global__ void __launch_bounds__(kSrThreads) sr_solve_kernel(SrArgs a) {
   // first solve
   for (int e = tid; e < nn1; e += kSrThreads) x[e] = sr_from<V>(rhs[perm[e / n1] * n1 + e % n1]);
   __syncthreads();
-  sr_solve_lu(n, n1, lu, x);
+  sr_solve_lu<false>(n, n1, lu, x);
   float loc = 0.0f;
   for (int e = tid; e < nn1; e += kSrThreads) {
     w[e] = sr_to64(x[e]);
@@ -633,11 +718,11 @@ __global__ void __launch_bounds__(kSrThreads) sr_solve_kernel(SrArgs a) {
     if constexpr (kDF) {
       for (int e = tid; e < nn1; e += kSrThreads) sr_split(w[e], wh[e], wlo[e]);
       __syncthreads();
-      for (int e = tid; e < nn1; e += kSrThreads) {
-        const int i = e / n1, c = e % n1;
-        sw[e] = sr_df_dot<false>(a.S0h + fo + i * n, a.S0l + fo + i * n, 1, wh + c, wlo + c, n1, n);
-        if (tnz) r[e] = sr_df_dot<false>(a.Th + fo + i * n, a.Tl + fo + i * n, 1, wh + c, wlo + c, n1, n);
-      }
+      sr_rows(nn1, [&](int e) { return sr_df_dot<false>(a.S0q + fo + e / n1 * n, wh + e % n1, wlo + e % n1, n1, n); },
+              [&](int e, double2 v) { sw[e] = v; });
+      if (tnz)
+        sr_rows(nn1, [&](int e) { return sr_df_dot<false>(a.Tq + fo + e / n1 * n, wh + e % n1, wlo + e % n1, n1, n); },
+                [&](int e, double2 v) { r[e] = v; });
     } else {
       for (int e = tid; e < nn1; e += kSrThreads) {
         const int i = e / n1, c = e % n1;
@@ -664,7 +749,7 @@ __global__ void __launch_bounds__(kSrThreads) sr_solve_kernel(SrArgs a) {
     __syncthreads();
     for (int e = tid; e < nn1; e += kSrThreads) x[e] = sr_from<V>(r[perm[e / n1] * n1 + e % n1]);
     __syncthreads();
-    sr_solve_lu(n, n1, lu, x);
+    sr_solve_lu<false>(n, n1, lu, x);
     float dl = 0.0f, wl = 0.0f;
     for (int e = tid; e < nn1; e += kSrThreads) {
       const double2 d = sr_to64(x[e]);
@@ -710,25 +795,36 @@ __global__ void __launch_bounds__(kSrThreads) sr_solve_kernel(SrArgs a) {
       for (int e = tid; e < nn1; e += kSrThreads) wh[e] = make_float2((float)w[e].x, (float)w[e].y);
       __syncthreads();
     }
-    for (int e = tid; e < n1 * a.L; e += kSrThreads) {
-      const int c = e / a.L, l = e % a.L;
-      double2 bl = make_double2(0.0, 0.0);
+    // nn1 points at a time; the FP32 form's field values through sw, idle by now
+    for (int p0 = 0; p0 < n1 * a.L; p0 += nn1) {
+      const int pc = min(nn1, n1 * a.L - p0);
       if constexpr (kDF) {
-        const float2* fr = a.fl32 + ((int64_t)f * a.L + l) * n;
-        float2 b32 = make_float2(0.f, 0.f);
-        for (int k = 0; k < n; ++k) b32 = sr_add(b32, sr_mul(fr[k], wh[k * n1 + c]));
-        bl = make_double2(b32.x, b32.y);
-      } else {
-        const double2* fr = a.field + ((int64_t)f * a.P + a.loss_idx[l]) * n;
-        for (int k = 0; k < n; ++k) bl = sr_add(bl, sr_mul(fr[k], w[k * n1 + c]));
+        sr_rows(pc,
+                [&](int e) {
+                  const int c = (p0 + e) / a.L, l = (p0 + e) % a.L;
+                  return sr_f32_dot<false>(a.fl32 + ((int64_t)f * a.L + l) * n, [&](int k) { return wh[k * n1 + c]; }, n);
+                },
+                [&](int e, float2 v) { sw[e] = make_double2(v.x, v.y); });
+        __syncthreads();
       }
-      const int64_t ti = ((int64_t)f * n1 + c) * a.L + l;
-      if (a.loss_offset) bl = sr_add(bl, a.loss_offset[ti]);
-      if (a.loss_weight) {
-        bl.x *= a.loss_weight[ti];
-        bl.y *= a.loss_weight[ti];
+      for (int e = p0 + tid; e < p0 + pc; e += kSrThreads) {
+        const int c = e / a.L, l = e % a.L;
+        double2 bl = make_double2(0.0, 0.0);
+        if constexpr (kDF) {
+          bl = sw[e - p0];
+        } else {
+          const double2* fr = a.field + ((int64_t)f * a.P + a.loss_idx[l]) * n;
+          for (int k = 0; k < n; ++k) bl = sr_add(bl, sr_mul(fr[k], w[k * n1 + c]));
+        }
+        const int64_t ti = ((int64_t)f * n1 + c) * a.L + l;
+        if (a.loss_offset) bl = sr_add(bl, a.loss_offset[ti]);
+        if (a.loss_weight) {
+          bl.x *= a.loss_weight[ti];
+          bl.y *= a.loss_weight[ti];
+        }
+        acc += sr_point_value(a.loss_mode, bl, a.target + ti * tw);
       }
-      acc += sr_point_value(a.loss_mode, bl, a.target + ti * tw);
+      if constexpr (kDF) __syncthreads();  // sw is written again
     }
     acc = sr_block_sum(acc, red);
     if (tid == 0) a.loss_part[g] = acc;
@@ -812,16 +908,23 @@ __global__ void __launch_bounds__(kSrThreads) sr_adjoint_kernel(SrArgs a) {
     const double gl = a.grad_loss[b] / a.norm;
     const int tw = a.loss_mode == 0 ? 1 : 2;
     double2* Gs = r;  // [n1][chunk]
-    for (int l0 = 0; l0 < a.L; l0 += kSrLossChunk) {
-      const int lc = min(kSrLossChunk, a.L - l0);
+    const int chunk = max(kSrLossChunk, n);  // what r holds
+    for (int l0 = 0; l0 < a.L; l0 += chunk) {
+      const int lc = min(chunk, a.L - l0);
+      if constexpr (kDF) {
+        sr_rows(n1 * lc,
+                [&](int e) {
+                  return sr_f32_dot<false>(a.fl32 + ((int64_t)f * a.L + l0 + e % lc) * n,
+                                           [&](int k) { return bh[k * n1 + e / lc]; }, n);
+                },
+                [&](int e, float2 v) { Gs[e / lc * chunk + e % lc] = make_double2(v.x, v.y); });
+        __syncthreads();
+      }
       for (int e = tid; e < n1 * lc; e += kSrThreads) {
         const int c = e / lc, l = l0 + e % lc;
         double2 bl = make_double2(0.0, 0.0);
         if constexpr (kDF) {
-          const float2* fr = a.fl32 + ((int64_t)f * a.L + l) * n;
-          float2 b32 = make_float2(0.f, 0.f);
-          for (int k = 0; k < n; ++k) b32 = sr_add(b32, sr_mul(fr[k], bh[k * n1 + c]));
-          bl = make_double2(b32.x, b32.y);
+          bl = Gs[c * chunk + (e % lc)];
         } else {
           const double2* fr = a.field + ((int64_t)f * a.P + a.loss_idx[l]) * n;
           for (int k = 0; k < n; ++k) bl = sr_add(bl, sr_mul(fr[k], w[k * n1 + c]));
@@ -837,27 +940,26 @@ __global__ void __launch_bounds__(kSrThreads) sr_adjoint_kernel(SrArgs a) {
         double2 G;
         if constexpr (kDF) G = sr_point_grad_f(a.loss_mode, bl, a.target + ti * tw);
         else sr_point_loss(a.loss_mode, bl, a.target + ti * tw, &G);
-        Gs[c * kSrLossChunk + (e % lc)] = make_double2(G.x * gl * wl, G.y * gl * wl);
+        Gs[c * chunk + (e % lc)] = make_double2(G.x * gl * wl, G.y * gl * wl);
       }
       __syncthreads();
-      for (int e = tid; e < nn1; e += kSrThreads) {
-        const int k = e / n1, c = e % n1;
-        double2 acc = gw[e];
-        if constexpr (kDF) {
-          float2 a32 = make_float2(0.f, 0.f);
-          for (int q = 0; q < lc; ++q) {
-            const double2 gq = Gs[c * kSrLossChunk + q];
-            a32 = sr_add(a32, sr_mul(sr_conj(a.fl32[((int64_t)f * a.L + l0 + q) * n + k]),
-                                     make_float2((float)gq.x, (float)gq.y)));
-          }
-          acc = sr_add(acc, make_double2(a32.x, a32.y));
-        } else {
+      if constexpr (kDF) {
+        sr_rows(nn1,
+                [&](int e) {
+                  return sr_f32_dot<true>(a.flT + ((int64_t)f * n + e / n1) * a.L + l0,
+                                          [&](int q) { return sr_from<float2>(Gs[e % n1 * chunk + q]); }, lc);
+                },
+                [&](int e, float2 v) { gw[e] = sr_add(gw[e], make_double2(v.x, v.y)); });
+      } else {
+        for (int e = tid; e < nn1; e += kSrThreads) {
+          const int k = e / n1, c = e % n1;
+          double2 acc = gw[e];
           for (int q = 0; q < lc; ++q) {
             const double2 fv = a.field[((int64_t)f * a.P + a.loss_idx[l0 + q]) * n + k];
-            acc = sr_add(acc, sr_mul(sr_conj(fv), Gs[c * kSrLossChunk + q]));
+            acc = sr_add(acc, sr_mul(sr_conj(fv), Gs[c * chunk + q]));
           }
+          gw[e] = acc;
         }
-        gw[e] = acc;
       }
       __syncthreads();
     }
@@ -877,7 +979,7 @@ __global__ void __launch_bounds__(kSrThreads) sr_adjoint_kernel(SrArgs a) {
   // Lambda = A^-H g_W
   for (int e = tid; e < nn1; e += kSrThreads) x[e] = sr_from<V>(gw[e]);
   __syncthreads();
-  sr_solve_lu_h(n, n1, lu, x);
+  sr_solve_lu<true>(n, n1, lu, x);
   float loc = 0.0f;
   for (int e = tid; e < nn1; e += kSrThreads) {
     const int i = e / n1, c = e % n1;
@@ -901,26 +1003,30 @@ __global__ void __launch_bounds__(kSrThreads) sr_adjoint_kernel(SrArgs a) {
       }
     }
     __syncthreads();
-    for (int e = tid; e < nn1; e += kSrThreads) {
-      const int i = e / n1, c = e % n1;
-      double2 acc = lam[e];
-      if constexpr (kDF) {
-        // column i of S0 (and T): conj(S0[j][i]) at j n + i
-        acc = sr_sub(acc, sr_df_dot<true>(a.S0h + fo + i, a.S0l + fo + i, n, ah + c, al + c, n1, n));
-        if (tnz)
-          acc = sr_sub(acc, sr_df_dot<true>(a.Th + fo + i, a.Tl + fo + i, n, bh + c, bl2 + c, n1, n));
-      } else {
+    if constexpr (kDF) {  // row i of S0^H (and T^H): conj of row i of the transpose
+      sr_rows(nn1,
+              [&](int e) {
+                double2 acc = sr_df_dot<true>(a.S0t + fo + e / n1 * n, ah + e % n1, al + e % n1, n1, n);
+                if (tnz)
+                  acc = sr_add(acc, sr_df_dot<true>(a.Tt + fo + e / n1 * n, bh + e % n1, bl2 + e % n1, n1, n));
+                return acc;
+              },
+              [&](int e, double2 v) { r[e] = sr_sub(gw[e], sr_sub(lam[e], v)); });
+    } else {
+      for (int e = tid; e < nn1; e += kSrThreads) {
+        const int i = e / n1, c = e % n1;
+        double2 acc = lam[e];
         for (int j = 0; j < n; ++j) {
           acc = sr_sub(acc, sr_mul(sr_conj(S0f[j * n + i]), y[j * n1 + c]));
           if (tnz) acc = sr_sub(acc, sr_mul(sr_conj(Tf[j * n + i]), lam[j * n1 + c]));
         }
+        r[e] = sr_sub(gw[e], acc);
       }
-      r[e] = sr_sub(gw[e], acc);
     }
     __syncthreads();
     for (int e = tid; e < nn1; e += kSrThreads) x[e] = sr_from<V>(r[e]);
     __syncthreads();
-    sr_solve_lu_h(n, n1, lu, x);
+    sr_solve_lu<true>(n, n1, lu, x);
     float dl = 0.0f, ll = 0.0f;
     for (int e = tid; e < nn1; e += kSrThreads) {
       const int i = e / n1, c = e % n1;
@@ -949,11 +1055,12 @@ __global__ void __launch_bounds__(kSrThreads) sr_adjoint_kernel(SrArgs a) {
     for (int e = tid; e < nn1; e += kSrThreads) sr_split(w[e], bh[e], bl2[e]);
     __syncthreads();
   }
-  for (int e = tid; e < nn1; e += kSrThreads) {
-    const int i = e / n1, c = e % n1;
-    if constexpr (kDF) {
-      sw[e] = sr_df_dot<false>(a.S0h + fo + i * n, a.S0l + fo + i * n, 1, bh + c, bl2 + c, n1, n);
-    } else {
+  if constexpr (kDF) {
+    sr_rows(nn1, [&](int e) { return sr_df_dot<false>(a.S0q + fo + e / n1 * n, bh + e % n1, bl2 + e % n1, n1, n); },
+            [&](int e, double2 v) { sw[e] = v; });
+  } else {
+    for (int e = tid; e < nn1; e += kSrThreads) {
+      const int i = e / n1, c = e % n1;
       double2 acc = make_double2(0.0, 0.0);
       for (int j = 0; j < n; ++j) acc = sr_add(acc, sr_mul(S0f[i * n + j], w[j * n1 + c]));
       sw[e] = acc;
@@ -1046,17 +1153,27 @@ __global__ void sr_const_kernel(int n0, int n1, const double2* __restrict__ S0,
   }
 }
 
-// hi/lo float pairs of a complex FP64 array (double-float operands of the residuals)
-__global__ void sr_split_kernel(int64_t n, const double2* __restrict__ src, float2* __restrict__ hi,
-                                float2* __restrict__ lo) {
+// complex FP64 matrices [.][n0][n0] in FP32, as (hi, lo) quadruples (double-float operands of the
+// residuals), and those transposed
+__global__ void sr_split_kernel(int64_t n, int n0, const double2* __restrict__ src, float2* __restrict__ hi,
+                                float4* __restrict__ quad, float4* __restrict__ tr) {
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n;
-       i += (int64_t)gridDim.x * blockDim.x)
-    sr_split(src[i], hi[i], lo[i]);
+       i += (int64_t)gridDim.x * blockDim.x) {
+    float2 h, l;
+    sr_split(src[i], h, l);
+    const float4 v = make_float4(h.x, h.y, l.x, l.y);
+    hi[i] = h;
+    quad[i] = v;
+    const int64_t f = i / (n0 * n0);
+    const int e = (int)(i - f * n0 * n0);
+    tr[f * n0 * n0 + e % n0 * n0 + e / n0] = v;
+  }
 }
 
-// the field's rows at the loss points in FP32, [F][L][n0]
+// the field's rows at the loss points in FP32, [F][L][n0] and [F][n0][L]
 __global__ void sr_lossrows_kernel(int F, int64_t P, int L, int n0, const double2* __restrict__ field,
-                                   const int64_t* __restrict__ loss_idx, float2* __restrict__ out) {
+                                   const int64_t* __restrict__ loss_idx, float2* __restrict__ out,
+                                   float2* __restrict__ tr) {
   const int64_t total = (int64_t)F * L * n0;
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < total;
        i += (int64_t)gridDim.x * blockDim.x) {
@@ -1065,6 +1182,7 @@ __global__ void sr_lossrows_kernel(int F, int64_t P, int L, int n0, const double
     const int f = (int)(fl / L), l = (int)(fl % L);
     const double2 v = field[((int64_t)f * P + loss_idx[l]) * n0 + k];
     out[i] = make_float2((float)v.x, (float)v.y);
+    tr[((int64_t)f * n0 + k) * L + l] = make_float2((float)v.x, (float)v.y);
   }
 }
 
@@ -1135,7 +1253,7 @@ __global__ void sr_rc_vjp_kernel(int64_t n_cfg, int F, int nL, const double* __r
 // host side: layouts, the internal per-frequency problem, launch sequences
 // ---------------------------------------------------------------------------------------
 struct SrBasisLayout {
-  size_t vport, vpoint, vfreq, vbasis, T, tflag, tabs, S0h, S0l, Th, Tl, fl32, total;
+  size_t vport, vpoint, vfreq, vbasis, T, tflag, tabs, S0h, Th, S0q, Tq, S0t, Tt, fl32, flT, total;
   BasisLayout vb;
 };
 
@@ -1189,10 +1307,13 @@ static SrBasisLayout sr_basis_layout(const mts_sparams* sp, mts_precision prec, 
   L.tflag = o; o += 256;
   L.tabs = o; o += align256(sizeof(SrTables));
   L.S0h = o; o += align256(8 * F * n0 * n0);
-  L.S0l = o; o += align256(8 * F * n0 * n0);
   L.Th = o; o += align256(8 * F * n0 * n0);
-  L.Tl = o; o += align256(8 * F * n0 * n0);
+  L.S0q = o; o += align256(16 * F * n0 * n0);
+  L.Tq = o; o += align256(16 * F * n0 * n0);
+  L.S0t = o; o += align256(16 * F * n0 * n0);
+  L.Tt = o; o += align256(16 * F * n0 * n0);
   L.fl32 = o; o += align256(8 * F * (size_t)sp->n_loss * n0);
+  L.flT = o; o += align256(8 * F * (size_t)sp->n_loss * n0);
   L.total = o;
   return L;
 }
@@ -1353,10 +1474,13 @@ static SrArgs sr_args(const mts_sparams* sp, mts_precision prec, const char* SB,
   a.loss_offset = reinterpret_cast<const double2*>(ev->loss_offset);
   a.tabs = reinterpret_cast<const SrTables*>(SB + BL.tabs);
   a.S0h = reinterpret_cast<const float2*>(SB + BL.S0h);
-  a.S0l = reinterpret_cast<const float2*>(SB + BL.S0l);
   a.Th = reinterpret_cast<const float2*>(SB + BL.Th);
-  a.Tl = reinterpret_cast<const float2*>(SB + BL.Tl);
+  a.S0q = reinterpret_cast<const float4*>(SB + BL.S0q);
+  a.Tq = reinterpret_cast<const float4*>(SB + BL.Tq);
+  a.S0t = reinterpret_cast<const float4*>(SB + BL.S0t);
+  a.Tt = reinterpret_cast<const float4*>(SB + BL.Tt);
   a.fl32 = reinterpret_cast<const float2*>(SB + BL.fl32);
+  a.flT = reinterpret_cast<const float2*>(SB + BL.flT);
   a.W = reinterpret_cast<double2*>(T + TL.W);
   a.lu = T + TL.lu;
   a.perm = reinterpret_cast<int32_t*>(T + TL.perm);
@@ -1426,21 +1550,23 @@ mts_status mts_sroute_build(const mts_sparams* sp, mts_precision prec, void* sba
   // double-float operands and FP32 loss rows of the FP32-factor kernels
   const int64_t nsq = (int64_t)F * n0 * n0;
   const unsigned sb = (unsigned)((nsq + 255) / 256 < 4096 ? (nsq + 255) / 256 : 4096);
-  sr_split_kernel<<<sb, 256, 0, st>>>(nsq, reinterpret_cast<const double2*>(sp->S0),
+  sr_split_kernel<<<sb, 256, 0, st>>>(nsq, n0, reinterpret_cast<const double2*>(sp->S0),
                                       reinterpret_cast<float2*>(SB + L.S0h),
-                                      reinterpret_cast<float2*>(SB + L.S0l));
+                                      reinterpret_cast<float4*>(SB + L.S0q),
+                                      reinterpret_cast<float4*>(SB + L.S0t));
   note_launch();
   if (sp->sc_const) {
-    sr_split_kernel<<<sb, 256, 0, st>>>(nsq, reinterpret_cast<const double2*>(SB + L.T),
+    sr_split_kernel<<<sb, 256, 0, st>>>(nsq, n0, reinterpret_cast<const double2*>(SB + L.T),
                                         reinterpret_cast<float2*>(SB + L.Th),
-                                        reinterpret_cast<float2*>(SB + L.Tl));
+                                        reinterpret_cast<float4*>(SB + L.Tq),
+                                        reinterpret_cast<float4*>(SB + L.Tt));
     note_launch();
   }
   if (sp->n_loss > 0) {
     const int64_t nl = (int64_t)F * sp->n_loss * n0;
     sr_lossrows_kernel<<<(unsigned)((nl + 255) / 256 < 4096 ? (nl + 255) / 256 : 4096), 256, 0, st>>>(
         F, sp->n_points, sp->n_loss, n0, reinterpret_cast<const double2*>(sp->field), sp->loss_idx,
-        reinterpret_cast<float2*>(SB + L.fl32));
+        reinterpret_cast<float2*>(SB + L.fl32), reinterpret_cast<float2*>(SB + L.flT));
     note_launch();
   }
   return sr_cuda(cudaGetLastError());
