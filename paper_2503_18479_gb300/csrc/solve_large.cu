@@ -350,6 +350,85 @@ __device__ inline void trailing_update(Cx<float>* __restrict__ A, int N, const i
   }
 }
 
+// Pivot steps of an FP32 panel of nb columns with its rows in registers: thread t holds rows
+// t, t + T, .. (N <= RPT T), so that a step reads nothing but the chosen row. Per step a warp finds
+// its largest |a|^2 (redux on the bits, the lowest lane of equals), its owner publishes the rest
+// of that row speculatively, and after the step's one barrier every thread takes the best
+// warp's row; keys and rows alternate by step parity. The steps on the panel in shared memory
+// (a read and a write of every entry) took 3700 cycles each for 1024 ports and 2000 for 128.
+// cand: [2][T / 32][16] entries of scratch. Leaves the panel and the pivot steps in shared memory.
+template <int T, int RPT>
+__device__ inline void panel_steps(Cx<float>* __restrict__ pan, Cx<float>* __restrict__ cand, int N, int nb,
+                                   int c0, int* __restrict__ pivstep, int* __restrict__ order, BlockRed* red) {
+  constexpr int NB = LargeCfg<float>::NB, W = T / 32;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, NP = N + 1;
+  Cx<float> v[RPT][NB];
+  bool own[RPT], open[RPT];
+#pragma unroll
+  for (int q = 0; q < RPT; ++q) {
+    const int r = tid + q * T;
+    own[q] = open[q] = r < N && pivstep[r] == N;
+#pragma unroll
+    for (int j = 0; j < NB; ++j) v[q][j] = own[q] ? pan[j * NP + r] : Cx<float>{0.0f, 0.0f};
+  }
+#pragma unroll
+  for (int kk = 0; kk < NB; ++kk) {
+    if (kk < nb) {
+      const int buf = kk & 1;
+      int key = -1, mine = 0;  // bits of a non-negative float order as integers
+#pragma unroll
+      for (int q = 0; q < RPT; ++q) {
+        float m = v[q][kk].x * v[q][kk].x + v[q][kk].y * v[q][kk].y;
+        if (!(m >= 0.0f)) m = 0.0f;  // NaN: still a candidate, so a row is always chosen
+        const int k = open[q] ? __float_as_int(m) : -1;
+        if (k > key) {
+          key = k;
+          mine = q;
+        }
+      }
+      const int best = __reduce_max_sync(0xffffffffu, key);
+      if (lane == __ffs(__ballot_sync(0xffffffffu, key == best)) - 1) {
+        red->pkeyf[buf][warp] = __int_as_float(best);
+        red->pidx[buf][warp] = tid + mine * T;
+        Cx<float>* c = cand + (buf * W + warp) * NB;
+#pragma unroll
+        for (int j = kk; j < NB; ++j) {
+          Cx<float> e = v[0][j];
+          if constexpr (RPT > 1)
+            if (mine == 1) e = v[1][j];
+          c[j] = e;
+        }
+      }
+      __syncthreads();
+      const int kq = lane < W ? __float_as_int(red->pkeyf[buf][lane]) : -1;
+      const int top = __reduce_max_sync(0xffffffffu, kq);
+      const int src = __ffs(__ballot_sync(0xffffffffu, kq == top)) - 1;
+      const int p = red->pidx[buf][src];
+      const Cx<float>* u = cand + (buf * W + src) * NB;
+      const Cx<float> piv = u[kk];
+#pragma unroll
+      for (int q = 0; q < RPT; ++q)
+        if (open[q]) {
+          if (tid + q * T == p) {
+            open[q] = false;
+            pivstep[p] = c0 + kk;
+          } else {
+            const Cx<float> l = cx_div(v[q][kk], piv);
+            v[q][kk] = l;
+#pragma unroll
+            for (int j = kk + 1; j < NB; ++j) cx_fnma(v[q][j], l, u[j]);
+          }
+        }
+      if (tid == 0) order[c0 + kk] = p;
+    }
+  }
+#pragma unroll
+  for (int q = 0; q < RPT; ++q)
+    if (own[q])
+#pragma unroll
+      for (int j = 0; j < NB; ++j) pan[j * NP + tid + q * T] = v[q][j];
+}
+
 // the same for 16 aligned bytes
 template <typename R>
 __device__ __forceinline__ void cp_async16(Cx<R>* dst, const Cx<R>* src) {
@@ -539,6 +618,11 @@ __global__ void __launch_bounds__(T, T == 128 ? 4 : (T == 256 ? 2 : 1)) solve_la
       // pivot steps with one barrier each: a thread reads and writes only its own rows of the
       // panel and their pivot steps, except the pivot row's entries, which its owner last
       // wrote before the barrier of this step's search
+      constexpr int RPT = T >= 512 ? 2 : 1;  // rows of a thread in the register form
+      if (kF && N <= RPT * T)
+        panel_steps<T, RPT>(reinterpret_cast<Cx<float>*>(pan), reinterpret_cast<Cx<float>*>(u12), N, nb,
+                            c0, pivstep, order, red);
+      else
       for (int kk = 0; kk < nb; ++kk) {
         int p;
         if constexpr (kF) {
