@@ -283,8 +283,8 @@ __device__ inline void outer_u_rows(Cx<float>* __restrict__ A, int N, const int*
 // 4.1e9 of 11.4e9 instructions on the ALU pipe, 46 % of the issue slots used). A tile's
 // multipliers are loaded into registers a tile ahead and put into the warp's own KB x 4 slots
 // of `lst`. src: the multiplier of row r and column m at src[r rs + m ms].
-template <int T, int KB>
-__device__ inline void trailing_update(Cx<float>* __restrict__ A, int N, const int* __restrict__ alist,
+template <int T, int KB, int CC>
+__device__ inline void trailing_tiles(Cx<float>* __restrict__ A, int N, const int* __restrict__ alist,
                                        int nact, int j0, const Cx<float>* __restrict__ src, int rs,
                                        int ms, const Cx<float>* __restrict__ ub, float4* __restrict__ lst) {
   constexpr int W = T / 32, CW = 128, NL = 4 * KB / 32;
@@ -304,13 +304,13 @@ __device__ inline void trailing_update(Cx<float>* __restrict__ A, int N, const i
     __syncwarp();  // every lane is done with the previous tile's multipliers
 #pragma unroll
     for (int i = 0; i < NL; ++i) buf[i * 32 + lane] = make_float4(-ln[i].x, -ln[i].x, ln[i].y, ln[i].y);
-    unsigned long long V[4][4];
+    unsigned long long V[4][CC];
 #pragma unroll
     for (int rr = 0; rr < 4; ++rr) {
       const bool okr = 4 * t4 + rr < nact;
       const Cx<float>* row = A + (int64_t)alist[okr ? 4 * t4 + rr : 0] * N;
 #pragma unroll
-      for (int cc = 0; cc < 4; ++cc) {
+      for (int cc = 0; cc < CC; ++cc) {
         const int j = jc + 32 * cc;
         V[rr][cc] = (okr && j < N) ? *reinterpret_cast<const unsigned long long*>(row + j) : 0ull;
       }
@@ -322,9 +322,9 @@ __device__ inline void trailing_update(Cx<float>* __restrict__ A, int N, const i
       ulonglong2 l[4];  // (-a, -a), (b, b)
 #pragma unroll
       for (int rr = 0; rr < 4; ++rr) l[rr] = *reinterpret_cast<const ulonglong2*>(buf + rr * KB + m);
-      unsigned long long P1[4], P2[4];
+      unsigned long long P1[CC], P2[CC];
 #pragma unroll
-      for (int cc = 0; cc < 4; ++cc) {
+      for (int cc = 0; cc < CC; ++cc) {
         const Cx<float> u = ub[m * CW + lane + 32 * cc];
         asm("mov.b64 %0, {%1,%2};" : "=l"(P1[cc]) : "f"(u.x), "f"(u.y));
         asm("mov.b64 %0, {%1,%2};" : "=l"(P2[cc]) : "f"(u.y), "f"(-u.x));
@@ -332,7 +332,7 @@ __device__ inline void trailing_update(Cx<float>* __restrict__ A, int N, const i
 #pragma unroll
       for (int rr = 0; rr < 4; ++rr)
 #pragma unroll
-        for (int cc = 0; cc < 4; ++cc) {
+        for (int cc = 0; cc < CC; ++cc) {
           asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(V[rr][cc]) : "l"(l[rr].y), "l"(P2[cc]));
           asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(V[rr][cc]) : "l"(l[rr].x), "l"(P1[cc]));
         }
@@ -342,12 +342,24 @@ __device__ inline void trailing_update(Cx<float>* __restrict__ A, int N, const i
       if (4 * t4 + rr < nact) {
         Cx<float>* row = A + (int64_t)alist[4 * t4 + rr] * N;
 #pragma unroll
-        for (int cc = 0; cc < 4; ++cc) {
+        for (int cc = 0; cc < CC; ++cc) {
           const int j = jc + 32 * cc;
           if (j < N) *reinterpret_cast<unsigned long long*>(row + j) = V[rr][cc];
         }
       }
   }
+}
+
+// A chunk with at most 32 or 64 columns left takes one or two columns a lane instead of four:
+// 1000 systems of 80 ports (forward and a field backward) 589 -> 556 us. Not with 512 threads,
+// where the three forms together spill: 256 systems of 1024 ports 30.7 -> 31.1 ms.
+template <int T, int KB>
+__device__ inline void trailing_update(Cx<float>* __restrict__ A, int N, const int* __restrict__ alist,
+                                       int nact, int j0, const Cx<float>* __restrict__ src, int rs,
+                                       int ms, const Cx<float>* __restrict__ ub, float4* __restrict__ lst) {
+  if (T < 512 && N - j0 <= 32) trailing_tiles<T, KB, 1>(A, N, alist, nact, j0, src, rs, ms, ub, lst);
+  else if (T < 512 && N - j0 <= 64) trailing_tiles<T, KB, 2>(A, N, alist, nact, j0, src, rs, ms, ub, lst);
+  else trailing_tiles<T, KB, 4>(A, N, alist, nact, j0, src, rs, ms, ub, lst);
 }
 
 // Pivot steps of an FP32 panel of nb columns with its rows in registers: thread t holds rows
