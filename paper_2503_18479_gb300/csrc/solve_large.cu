@@ -882,7 +882,7 @@ __global__ void __launch_bounds__(T, T == 128 ? 4 : (T == 256 ? 2 : 1)) solve_la
   // u ^ (r % 8) so that threads of consecutive rows read different banks. Copies of one entry
   // per lane and row fetched every 32-byte sector four times. ----
   Cx<R>* const stg = pan;  // [N][128 bytes]
-  Cx<R>* const dstg = u12;  // [NB][32]
+  Cx<R>* const dstg = u12;  // [2][NB][32], by step parity
   constexpr int UE = 16 / (int)sizeof(Cx<R>);  // entries of a 16-byte unit
   const bool unit16 = (N & 1) == 0 && (reinterpret_cast<uintptr_t>(A) & 15) == 0;
   auto stg_at = [&](int r, int m) -> Cx<R>* { return stg + r * NB + ((m / UE) ^ (r & 7)) * UE + m % UE; };
@@ -910,12 +910,24 @@ __global__ void __launch_bounds__(T, T == 128 ? 4 : (T == 256 ? 2 : 1)) solve_la
             }
           }
         }
+        asm volatile("cp.async.commit_group;" ::: "memory");
+      }
+    };
+    // warp 0's rows of the diagonal block of a step, a whole step ahead: its products begin the
+    // step, those of the rows above come after its barrier, so that the rows' copies have the
+    // diagonal's products to arrive in. With both asked for after the step before, a step of 80
+    // ports took 4000 cycles, most of them L2 latency. (This and twice to four times the
+    // loads of M and H in flight in the residual and the objective: 256 systems of 1024 ports
+    // 30.7 -> 28.8 ms, the 128-port class of 300 ragged structures 408 -> 380 us.)
+    auto fetch_diag = [&](int c0, bool fwd) {
+      if constexpr (!SA) {
+        const int nb = min(NB, N - c0);
         if (warp == 0 && lane < nb) {
           const int pi = order[c0 + lane];
+          Cx<R>* d = dstg + ((c0 / NB + fwd) & 1) * NB * 32 + lane;
 #pragma unroll
           for (int m = 0; m < NB; ++m)  // W_b row (forward), V_b row (back)
-            if (fwd ? m < lane : (m >= lane && m < nb))
-              cp_async_elem(dstg + m * 32 + lane, A + (int64_t)pi * N + c0 + m);
+            if (fwd ? m < lane : (m >= lane && m < nb)) cp_async_elem(d + m * 32, A + (int64_t)pi * N + c0 + m);
         }
         asm volatile("cp.async.commit_group;" ::: "memory");
       }
@@ -940,14 +952,18 @@ __global__ void __launch_bounds__(T, T == 128 ? 4 : (T == 256 ? 2 : 1)) solve_la
       wv[r] = v;
     };
     // entry m of this lane's diagonal row (the matrix itself when it is in shared memory)
-    auto diag_elem = [&](int c0, int pi, int m) -> Cx<R> {
+    auto diag_elem = [&](int c0, bool fwd, int pi, int m) -> Cx<R> {
       if constexpr (SA) return A[(int64_t)pi * N + c0 + m];
-      else return dstg[m * 32 + lane];
+      else return dstg[((c0 / NB + fwd) & 1) * NB * 32 + m * 32 + lane];
     };
+    // copy groups of a thread in order: diag(step), rows(step), diag(step + 1), rows(step + 1), ..
+    fetch_diag(0, true);
     fetch(0, true);
     __syncthreads();
     for (int c0 = 0; c0 < N; c0 += NB) {  // forward: L y = P rhs
       const int nb = min(NB, N - c0);
+      if (c0 + NB < N) fetch_diag(c0 + NB, true);
+      else fetch_diag(last, false);
       if (warp == 0) {
         Cx<R> wi = {0, 0};
         int pi = 0;
@@ -955,14 +971,15 @@ __global__ void __launch_bounds__(T, T == 128 ? 4 : (T == 256 ? 2 : 1)) solve_la
           pi = order[c0 + lane];
           wi = wv[pi];
         }
-        if constexpr (!SA) asm volatile("cp.async.wait_all;" ::: "memory");
+        if constexpr (!SA) asm volatile("cp.async.wait_group 2;" ::: "memory");
+        __syncwarp();
         // y_b = W_b w_b (unit diagonal): products of the block's original values
         const Cx<R> w0 = wi;
 #pragma unroll
         for (int m = 0; m < NB; ++m) {
           const Cx<R> wm = {__shfl_sync(0xffffffffu, w0.x, m), __shfl_sync(0xffffffffu, w0.y, m)};
           if (lane > m && lane < nb) {  // wi += W_im w_m
-            const Cx<R> l = diag_elem(c0, pi, m);
+            const Cx<R> l = diag_elem(c0, true, pi, m);
             wi.x = fma(l.x, wm.x, fma(-l.y, wm.y, wi.x));
             wi.y = fma(l.x, wm.y, fma(l.y, wm.x, wi.y));
           }
@@ -971,7 +988,7 @@ __global__ void __launch_bounds__(T, T == 128 ? 4 : (T == 256 ? 2 : 1)) solve_la
         if (lane < nb) wv[pi] = wi;
       }
       __syncthreads();
-      if constexpr (!SA) asm volatile("cp.async.wait_all;" ::: "memory");
+      if constexpr (!SA) asm volatile("cp.async.wait_group 1;" ::: "memory");
       __syncwarp();  // the warp's copies, by whichever of its lanes
       for (int r = tid; r < N; r += T)
         if (pivstep[r] >= c0 + nb) row_update(r, c0, nb);
@@ -981,6 +998,8 @@ __global__ void __launch_bounds__(T, T == 128 ? 4 : (T == 256 ? 2 : 1)) solve_la
     }
     for (int c0 = last; c0 >= 0; c0 -= NB) {  // back: U x = y
       const int nb = min(NB, N - c0);
+      if (c0 > 0) fetch_diag(c0 - NB, false);
+      else if constexpr (!SA) asm volatile("cp.async.commit_group;" ::: "memory");
       if (warp == 0) {
         Cx<R> wi = {0, 0};
         int pi = 0;
@@ -988,7 +1007,8 @@ __global__ void __launch_bounds__(T, T == 128 ? 4 : (T == 256 ? 2 : 1)) solve_la
           pi = order[c0 + lane];
           wi = wv[pi];
         }
-        if constexpr (!SA) asm volatile("cp.async.wait_all;" ::: "memory");
+        if constexpr (!SA) asm volatile("cp.async.wait_group 2;" ::: "memory");
+        __syncwarp();
         // x_b = V_b y_b: products of the block's values
         const Cx<R> y0 = wi;
         wi = {0, 0};
@@ -996,7 +1016,7 @@ __global__ void __launch_bounds__(T, T == 128 ? 4 : (T == 256 ? 2 : 1)) solve_la
         for (int m = 0; m < NB; ++m) {
           const Cx<R> ym = {__shfl_sync(0xffffffffu, y0.x, m), __shfl_sync(0xffffffffu, y0.y, m)};
           if (m >= lane && m < nb && lane < nb) {  // wi += V_im y_m
-            const Cx<R> u = diag_elem(c0, pi, m);
+            const Cx<R> u = diag_elem(c0, false, pi, m);
             wi.x = fma(u.x, ym.x, fma(-u.y, ym.y, wi.x));
             wi.y = fma(u.x, ym.y, fma(u.y, ym.x, wi.y));
           }
@@ -1005,7 +1025,7 @@ __global__ void __launch_bounds__(T, T == 128 ? 4 : (T == 256 ? 2 : 1)) solve_la
         if (lane < nb) wv[pi] = wi;
       }
       __syncthreads();
-      if constexpr (!SA) asm volatile("cp.async.wait_all;" ::: "memory");
+      if constexpr (!SA) asm volatile("cp.async.wait_group 1;" ::: "memory");
       __syncwarp();
       for (int r = tid; r < N; r += T)
         if (pivstep[r] < c0) row_update(r, c0, nb);
@@ -1039,7 +1059,7 @@ __global__ void __launch_bounds__(T, T == 128 ? 4 : (T == 256 ? 2 : 1)) solve_la
         __syncthreads();
         for (int r = tid; r < N; r += T) {  // residual sv - A xk, M x in double-float
           float shx = 0.f, slx = 0.f, shy = 0.f, sly = 0.f;
-#pragma unroll 4
+#pragma unroll 8
           for (int j = 0; j < N; ++j) {
             const float mh = Mh[(int64_t)j * N + r], ml = Ml[(int64_t)j * N + r];  // column r
             const float2 ph = xh[j], pl = xl[j];
@@ -1157,7 +1177,7 @@ __global__ void __launch_bounds__(T, T == 128 ? 4 : (T == 256 ? 2 : 1)) solve_la
             // FP32 rows (the basis is FP32), double-float sums: N terms with cancellation
             // (sum |H x| / |b| reaches ~100 at N = 1024) need more than FP32 accumulation
             float hx = 0.f, lx = 0.f, hy = 0.f, ly = 0.f;
-#pragma unroll 4
+#pragma unroll 16
             for (int k = 0; k < N; ++k) {
               const float h = HlT32[(int64_t)k * Ls + l];  // lanes l read consecutively
               lg_df_acc(hx, lx, h, xh[k].x);
@@ -1201,7 +1221,7 @@ __global__ void __launch_bounds__(T, T == 128 ? 4 : (T == 256 ? 2 : 1)) solve_la
         for (int r = tid; r < N; r += T) {
           if constexpr (kF) {
             float hx = 0.f, lx = 0.f, hy = 0.f, ly = 0.f;
-#pragma unroll 4
+#pragma unroll 16
             for (int q = 0; q < lc; ++q) {
               const float h = Hl32[(int64_t)(c0 + q) * N + r];
               lg_df_acc(hx, lx, h, Gh[q].x);
