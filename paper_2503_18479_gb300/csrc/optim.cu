@@ -26,14 +26,15 @@ __global__ void adam_kernel(int64_t n, mts_adam o, double* __restrict__ C, doubl
   // What depends on the step alone is computed by one thread per CTA. The update is bound by
   // the FP64 pipe (1/76 of the FP32 rate): with both powers, the division and the square root
   // in every thread the step took 112 us for 262,144 parameters.
-  __shared__ double s_c[2];  // lr / (1 - b1^t), sqrt(1 - b2^t)
+  __shared__ double s_c[2];  // lr root2 / (1 - b1^t) and eps root2, root2 = sqrt(1 - b2^t)
   const int64_t t = step[0] + 1;
   if (threadIdx.x == 0) {
-    s_c[0] = o.lr / (1.0 - pow(o.beta1, (double)t));
-    s_c[1] = sqrt(1.0 - pow(o.beta2, (double)t));
+    const double root2 = sqrt(1.0 - pow(o.beta2, (double)t));
+    s_c[0] = o.lr / (1.0 - pow(o.beta1, (double)t)) * root2;
+    s_c[1] = o.eps * root2;
   }
   __syncthreads();
-  const double lr_t = s_c[0], root2 = s_c[1];
+  const double lr_t = s_c[0], eps_t = s_c[1];
   const double c_mid = 0.5 * (o.c_max + o.c_min), c_half = 0.5 * (o.c_max - o.c_min);
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n;
        i += (int64_t)gridDim.x * blockDim.x) {
@@ -48,8 +49,8 @@ __global__ void adam_kernel(int64_t n, mts_adam o, double* __restrict__ C, doubl
     const double vi = o.beta2 * v[i] + (1.0 - o.beta2) * gi * gi;
     m[i] = mi;
     v[i] = vi;
-    const double denom = sqrt(vi) / root2 + o.eps;
-    th = th - lr_t * (mi / denom);
+    // lr_t mi / (sqrt(vi) / root2 + eps) with one division
+    th = th - lr_t * mi / (sqrt(vi) + eps_t);
     if (o.projection == MTS_PROJ_TANH) {
       u[i] = th;
       C[i] = c_mid + c_half * tanh(th);
