@@ -10,6 +10,7 @@
 
 #include "common.cuh"
 #include "kernels.h"
+#include "solve_common.cuh"
 
 namespace mts {
 
@@ -171,29 +172,29 @@ constexpr int kSimtHPitch = SimtCfg<float>::KC + 4;  // floats per staged H row 
 template <int SC>
 __device__ inline void simt_accumulate_f2(const float* __restrict__ hr, const float* __restrict__ sI,
                                           int kn, unsigned long long (&acc)[kSimtSys]) {
+  // (unrolled over all 64 k, the three sizes did not fit in the instruction cache: a quarter of
+  // the stall cycles were instruction fetches)
+#pragma unroll 4
+  for (int k4 = 0; k4 < kn; k4 += 4) {  // kn is a multiple of 4
+    const float4 h4 = *reinterpret_cast<const float4*>(hr + k4);
+    const float hv[4] = {h4.x, h4.y, h4.z, h4.w};
 #pragma unroll
-  for (int k4 = 0; k4 < SimtCfg<float>::KC; k4 += 4) {
-    if (k4 < kn) {  // kn is a multiple of 4
-      const float4 h4 = *reinterpret_cast<const float4*>(hr + k4);
-      const float hv[4] = {h4.x, h4.y, h4.z, h4.w};
+    for (int e = 0; e < 4; ++e) {
+      unsigned long long hh;
+      asm("mov.b64 %0, {%1,%1};" : "=l"(hh) : "f"(hv[e]));
+      const ulonglong2* ik = reinterpret_cast<const ulonglong2*>(sI + 2 * kSimtSys * (k4 + e));
 #pragma unroll
-      for (int e = 0; e < 4; ++e) {
-        unsigned long long hh;
-        asm("mov.b64 %0, {%1,%1};" : "=l"(hh) : "f"(hv[e]));
-        const ulonglong2* ik = reinterpret_cast<const ulonglong2*>(sI + 2 * kSimtSys * (k4 + e));
-#pragma unroll
-        for (int i2 = 0; i2 < SC / 2; ++i2) {
-          const ulonglong2 c = ik[i2];
-          asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(acc[2 * i2]) : "l"(hh), "l"(c.x));
-          asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(acc[2 * i2 + 1]) : "l"(hh), "l"(c.y));
-        }
+      for (int i2 = 0; i2 < SC / 2; ++i2) {
+        const ulonglong2 c = ik[i2];
+        asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(acc[2 * i2]) : "l"(hh), "l"(c.x));
+        asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(acc[2 * i2 + 1]) : "l"(hh), "l"(c.y));
       }
     }
   }
 }
 
 template <typename T>
-__global__ void __launch_bounds__(kSimtPts) superpose_simt_kernel(SuperposeArgs a) {
+__global__ void __launch_bounds__(kSimtPts, sizeof(T) == 4 ? 5 : 1) superpose_simt_kernel(SuperposeArgs a) {
   constexpr int KC = SimtCfg<T>::KC, VEC = SimtCfg<T>::VEC;
   using C2 = typename SimtCfg<T>::C2;
   using V = typename SimtCfg<T>::V;
@@ -261,7 +262,7 @@ __global__ void __launch_bounds__(kSimtPts) superpose_simt_kernel(SuperposeArgs 
           const int kn = min(KC, N - k0);
           const int q4 = kn / 4;  // 16-byte pieces per row
           for (int e = t; e < kSimtPts * q4; e += kSimtPts) {
-            const int r = e / q4, c = e - r * q4;
+            const int r = q4 == KC / 4 ? e / (KC / 4) : e / q4, c = e - r * q4;
             const uint32_t dst = (uint32_t)__cvta_generic_to_shared(sH + r * HP + 4 * c);
             const float* src = r < rows ? hblk + (int64_t)r * N + k0 + 4 * c : hblk;
             asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src),
@@ -270,16 +271,25 @@ __global__ void __launch_bounds__(kSimtPts) superpose_simt_kernel(SuperposeArgs 
           }
           asm volatile("cp.async.commit_group;" ::: "memory");
           if (stage_I) {
-            for (int e = t; e < kn * kSimtSys; e += kSimtPts) {
-              const int k = e / kSimtSys, i = e - k * kSimtSys;
-              float re = 0.0f, im = 0.0f;
-              if (i < nsv) {
-                const double* Ip = a.I + s_ioff[i] + 2 * (k0 + k);
-                re = (float)Ip[0];
-                im = (float)Ip[1];
-              }
-              sI[2 * (k * kSimtSys + i)] = re;
-              sI[2 * (k * kSimtSys + i) + 1] = im;
+            // a thread stages every eighth k of one system, all its loads in flight, converted off
+            // the FP64 pipe (one at a time, each waited for L2 and the tile's copies for all
+            // eight; with the loop above rolled, 300 ragged structures 233 -> 195 us, 6000 of them
+            // 2.70 -> 2.25 ms)
+            constexpr int U = KC * kSimtSys / kSimtPts;
+            const int i = t % kSimtSys;
+            const double2* Ip = reinterpret_cast<const double2*>(a.I + s_ioff[i]) + k0;
+            double2 v[U];
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+              const int k = t / kSimtSys + u * (kSimtPts / kSimtSys);
+              v[u] = i < nsv && k < kn ? Ip[k] : make_double2(0.0, 0.0);
+            }
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+              const int k = t / kSimtSys + u * (kSimtPts / kSimtSys);
+              if (k < kn)
+                *reinterpret_cast<float2*>(sI + 2 * (k * kSimtSys + i)) =
+                    make_float2(df_from(v[u].x).h, df_from(v[u].y).h);
             }
           }
           asm volatile("cp.async.wait_all;" ::: "memory");
