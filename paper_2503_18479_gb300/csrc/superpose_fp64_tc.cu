@@ -47,19 +47,12 @@ constexpr int kCols = 64;                             // columns of a tile: kSys
 constexpr int kSys = kCols / 2;
 constexpr uint32_t kABytes = kTileP * kChunkK * 2;    // one digit of the point tile: 16 KB
 constexpr uint32_t kBBytes = kCols * kChunkK * 2;     // one digit of the column tile: 8 KB
+constexpr int kWin = 4;                               // groups of a window: N = 256
 constexpr int kRows = kTileP / (kThreads / 32);       // rows of H per warp
 constexpr int kSysWarp = kSys / (kThreads / 32);      // systems per warp
 
-// kind::f16, A = B = bf16, D = f32, both K-major, M = 128, N = 64 n
-__device__ inline void mma_n64(uint32_t d, uint64_t ad, uint64_t bd, int n, uint32_t accum) {
-  const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(8 * n) << 17) | ((128u >> 4) << 24);
-  asm volatile(
-      "{\n\t.reg .pred p;\n\t"
-      "setp.ne.b32 p, %4, 0;\n\t"
-      "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(d),
-      "l"(ad), "l"(bd), "r"(idesc), "r"(accum)
-      : "memory");
-}
+// kind::f16, A = B = bf16, D = f32, both K-major, M = 128, N = kWin kCols
+constexpr uint32_t kIdescWin = (kIdesc & ~(0x3fu << 17)) | ((uint32_t)(kWin * kCols >> 3) << 17);
 
 __device__ inline void tmem_ld4(uint32_t taddr, float* v) {
   uint32_t* r = reinterpret_cast<uint32_t*>(v);
@@ -153,7 +146,8 @@ __global__ void __launch_bounds__(kThreads, 1) superpose_fp64_tc_kernel(Superpos
   extern __shared__ __align__(1024) unsigned char smem_dyn[];
   const uintptr_t sbase = (reinterpret_cast<uintptr_t>(smem_dyn) + 1023) & ~uintptr_t(1023);
   unsigned char* sA = reinterpret_cast<unsigned char*>(sbase);
-  unsigned char* sB = sA + kDigits * kABytes;
+  unsigned char* sZ = sA + kDigits * kABytes;  // images of zeros before those of the columns
+  unsigned char* sB = sZ + (kWin - 1) * kBBytes;
   uint64_t* bar = reinterpret_cast<uint64_t*>(sB + kDigits * kBBytes);  // MMAs of a turn done
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bar + 1);
   int* eA = reinterpret_cast<int*>(tmem_slot + 2);  // [2][128] row exponents, two point tiles in turn
@@ -168,6 +162,8 @@ __global__ void __launch_bounds__(kThreads, 1) superpose_fp64_tc_kernel(Superpos
   const bool vec = (N & 1) == 0;  // rows of H on 16-byte boundaries
   const int64_t u_begin = units * blockIdx.x / gridDim.x, u_end = units * (blockIdx.x + 1) / gridDim.x;
 
+  for (uint32_t o = 16 * t; o < (kWin - 1) * kBBytes; o += 16 * kThreads)
+    *reinterpret_cast<uint4*>(sZ + o) = make_uint4(0u, 0u, 0u, 0u);
   if (t == 0) {
     mbar_init(bar, 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -315,17 +311,19 @@ __global__ void __launch_bounds__(kThreads, 1) superpose_fp64_tc_kernel(Superpos
         tc_fence_after();
         const int ksteps = min(kChunkK / 16, (N - kc * kChunkK + 15) / 16);
         const uint32_t aA = smem_u32(sA), aB = smem_u32(sB);
-        // Digit i of the points with up to four digits j .. of the columns as one N = 256 MMA: the
-        // digits' images follow each other in shared memory as rows of one operand, and so do
-        // the accumulators of the groups i + j .. in tensor memory (12 MMAs a K step instead of
-        // 36 of N = 64, which took 106 cycles each whatever their N).
+        // Digit i of the points with four digits of the columns, those of the groups g .. g + 3, as
+        // one N = 256 MMA: the digits' images follow each other in shared memory as rows of
+        // one operand, and so do the groups' accumulators in tensor memory (12 MMAs a K step
+        // instead of 36 of N = 64, which take as long each). The images before digit 0 are
+        // zeros. MMAs are only sure to run in order on one accumulator and in one shape, so the
+        // two windows are fixed: with N = 64 to 256 at every group's base the same 12 took the
+        // same time.
         for (int kk = 0; kk < ksteps; ++kk)
-          for (int i = 0; i < kDigits; ++i)
-            for (int j = 0; j < kDigits - i; j += 4) {
-              const int n = min(4, kDigits - i - j);
-              mma_n64(tmem + (i + j) * kCols, make_desc(aA + i * kABytes) + (uint64_t)(kk * 2),
-                      make_desc(aB + j * kBBytes) + (uint64_t)(kk * 2), n, (i > 0 || kk > 0) ? 1u : 0u);
-            }
+          for (int g = 0; g < kDigits; g += kWin)
+            for (int i = 0; i < g + kWin; ++i)
+              mma_bf16(tmem + g * kCols, make_desc(aA + i * kABytes) + (uint64_t)(kk * 2),
+                       make_desc(aB + g * kBBytes - i * kBBytes) + (uint64_t)(kk * 2),
+                       (i > 0 || kk > 0) ? 1u : 0u, kIdescWin);
         mma_commit(bar);
       }
       prev_pt = pt;
@@ -348,7 +346,9 @@ __global__ void __launch_bounds__(kThreads, 1) superpose_fp64_tc_kernel(Superpos
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(512u) : "memory");
 }
 
-constexpr size_t kSmem = 1024 + kDigits * (size_t)(kABytes + kBBytes) + 16 + 8 + 4 * 2 * (kTileP + kCols);
+constexpr size_t kSmem = 1024 + kDigits * (size_t)kABytes + (kDigits + kWin - 1) * (size_t)kBBytes + 16 + 8 +
+                         4 * 2 * (kTileP + kCols);
+static_assert(kSmem <= 232448, "227 KB a CTA");
 
 }  // namespace oz
 
