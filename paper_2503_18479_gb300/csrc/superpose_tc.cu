@@ -413,13 +413,18 @@ constexpr int kResidentMax = 9;  // of them at most for the column tile
 // An MMA of M = 128 takes much the same time for N = 128 and N = 256, so the products of an A
 // piece with the first two B pieces go out as one MMA of N = 256: the pieces' tiles follow each
 // other in shared memory as the rows of one operand, and the second one's products have an
-// accumulator of their own, which the epilogue adds (783 -> 648 us for the 65,600 points below).
-// The A pieces come in the order 1, 2, 0, because the first of them starts both accumulators.
+// accumulator of their own, which the epilogue adds (65,600 points below: 783 -> 733 us).
+//
+// MMAs are only sure to run in order on one accumulator in one shape. So a unit's products of
+// N = 256 (every A piece with B pieces 0 and 1) go out first, and when they are done those of
+// N = 128: piece 0 with the third B piece, and the packed last chunk. The A tiles come as pieces 1
+// and 2 of every full chunk, then their pieces 0, whose slots are held until both shapes have
+// read them (at most three of five slots or more), then the last chunk. The wait itself costs
+// nothing (the bound is the latency of the point tiles, 16 KB each, over the ring's slots), the
+// held slots do: 651 us in the order of arrival against 733 us, 282 against 323 us for half the
+// columns at K = 104. A tile of zeros beside the third pieces, which makes their products N = 256 too, takes a
+// slot for good: 734 and 305 us, 534 against 513 us at K = 192.
 constexpr uint32_t kIdesc256 = (kIdesc & ~(0x3fu << 17)) | ((256u >> 3) << 17);
-
-__device__ __forceinline__ constexpr int a_piece(int npieces, int t) {
-  return npieces == 3 ? (t == 0 ? 1 : (t == 1 ? 2 : 0)) : 0;
-}
 
 // 16 KB tiles that one side of a unit takes
 __host__ __device__ inline int unit_tiles(int N, int nkc, int npieces) {
@@ -439,11 +444,13 @@ __global__ void __launch_bounds__(kThreads, 1) superpose_tc_resident_kernel(Supe
   uint64_t* tfull = bempty + kResidentMax;                                 // [2]
   uint64_t* tempty = tfull + 2;                                            // [2]
   uint64_t* mdone = tempty + 2;
-  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(mdone + 1);
+  uint64_t* wide = mdone + 1;  // a unit's products of N = 256 done
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(wide + 1);
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int nkc = a.uni.nkc, N = a.uni.N;
   const bool packed = tail_packed(N, NPIECE);
+  const int nfull = packed ? nkc - 1 : nkc;  // chunks with a tile per piece
   const int nB = unit_tiles(N, nkc, NPIECE), ring = kSlots - nB;
   unsigned char* sA = sB + nB * kTileBytes;
   const int64_t nptile = a.uni.nptile, nntile = a.uni.nntile;
@@ -457,6 +464,7 @@ __global__ void __launch_bounds__(kThreads, 1) superpose_tc_resident_kernel(Supe
       mbar_init(&tempty[i], 128);
     }
     mbar_init(mdone, 1);
+    mbar_init(wide, 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   if (warp == 1) {
@@ -489,8 +497,20 @@ __global__ void __launch_bounds__(kThreads, 1) superpose_tc_resident_kernel(Supe
           ++nb;
           b_chunks = 0;
         }
+        auto tile = [&](int q, int kc) {  // piece q of chunk kc of the point tile
+          ok = mbar_wait(&empty[slot], phase ^ 1u, err, 1);
+          if (!ok) return;
+          mbar_arrive_expect_tx(&full[slot], kTileBytes);
+          bulk_g2s(sA + slot * kTileBytes, Ab + ((size_t)(q * nptile + pt) * nkc + kc) * kTileBytes,
+                   kTileBytes, &full[slot]);
+          ++copies;
+          if (++slot == ring) {
+            slot = 0;
+            phase ^= 1u;
+          }
+        };
         for (int kc = 0; kc < nkc && ok; ++kc) {
-          const int np = packed && kc == nkc - 1 ? 1 : NPIECE;
+          const int np = kc == nfull ? 1 : NPIECE;
           if (fresh) {
             ok = mbar_wait(&bempty[kc], (uint32_t)nb & 1u, err, 1);
             if (!ok) break;
@@ -500,20 +520,10 @@ __global__ void __launch_bounds__(kThreads, 1) superpose_tc_resident_kernel(Supe
                        Bb + ((size_t)(q * nntile + nt) * nkc + kc) * kTileBytes, kTileBytes, &bfull[kc]);
             b_chunks = kc + 1;
           }
-          for (int i = 0; i < np; ++i) {
-            const int q = np == 1 ? 0 : a_piece(NPIECE, i);
-            ok = mbar_wait(&empty[slot], phase ^ 1u, err, 1);
-            if (!ok) break;
-            mbar_arrive_expect_tx(&full[slot], kTileBytes);
-            bulk_g2s(sA + slot * kTileBytes, Ab + ((size_t)(q * nptile + pt) * nkc + kc) * kTileBytes,
-                     kTileBytes, &full[slot]);
-            ++copies;
-            if (++slot == ring) {
-              slot = 0;
-              phase ^= 1u;
-            }
-          }
+          for (int q = NPIECE == 1 ? 0 : 1; q < np && ok; ++q) tile(q, kc);
         }
+        if constexpr (NPIECE == 3)
+          for (int kc = 0; kc < nkc && ok; ++kc) tile(0, kc);
       }
       // no copy may still be in flight when the CTA exits: the last use of every slot and chunk
       for (int i = 0; i < ring && i < copies; ++i)
@@ -527,75 +537,93 @@ __global__ void __launch_bounds__(kThreads, 1) superpose_tc_resident_kernel(Supe
     // ---------------- MMA issuer ----------------
     if (lane == 0) {
       int slot = 0, nb = 0, acc = 0;
-      uint32_t phase = 0, aphase = 0;
-      int64_t held = -1;
+      uint32_t phase = 0, aphase = 0, wphase = 0;
+      int64_t held_nt = -1;
       bool ok = true;
       for (int64_t u = u_begin; u < u_end && ok; ++u) {
         const int64_t nt = u / nptile;
-        const bool fresh = nt != held, last = u + 1 == u_end || (u + 1) / nptile != nt;
+        const bool fresh = nt != held_nt, last = u + 1 == u_end || (u + 1) / nptile != nt;
         if (fresh) {
-          held = nt;
+          held_nt = nt;
           ++nb;
         }
         ok = mbar_wait(&tempty[acc], aphase ^ 1u, err, 2);
         if (!ok) break;
         tc_fence_after();
         const uint32_t d_tmem = tmem_base + (uint32_t)acc * kAcc;
-        for (int kc = 0; kc < nkc && ok; ++kc) {
-          if (fresh) {
-            ok = mbar_wait(&bfull[kc], (uint32_t)(nb - 1) & 1u, err, 3);
-            if (!ok) break;
-          }
+        // K steps of the A tile in a slot with piece qb of chunk kc
+        auto steps = [&](int s, int kc, int qb, uint32_t idesc, bool first) {
           const int ksteps = min(kChunkK / 16, (N - kc * kChunkK + 15) / 16);
-          const uint32_t b0 = smem_u32(sB) + (uint32_t)(kc * NPIECE) * kTileBytes;
-          if (packed && kc == nkc - 1) {  // piece q is K step q of the one tile
-            ok = mbar_wait(&full[slot], phase, err, 3);
-            if (!ok) break;
-            tc_fence_after();
-            const uint64_t da = make_desc(smem_u32(sA) + (uint32_t)slot * kTileBytes), db = make_desc(b0);
+          const uint64_t da = make_desc(smem_u32(sA) + (uint32_t)s * kTileBytes);
+          const uint64_t db = make_desc(smem_u32(sB) + (uint32_t)(kc * NPIECE + qb) * kTileBytes);
 #pragma unroll
-            for (int qa = NPIECE - 1; qa >= 0; --qa)
-#pragma unroll
-              for (int qb = NPIECE - 1 - qa; qb >= 0; --qb)
-                mma_bf16(d_tmem, da + (uint64_t)(qa * 2), db + (uint64_t)(qb * 2),
-                         1u);
-            mma_commit(&empty[slot]);
-            if (++slot == ring) {
-              slot = 0;
-              phase ^= 1u;
+          for (int kk = 0; kk < kChunkK / 16; ++kk)
+            if (kk < ksteps)
+              mma_bf16(d_tmem, da + (uint64_t)(kk * 2), db + (uint64_t)(kk * 2), (!first || kk > 0) ? 1u : 0u,
+                       idesc);
+        };
+        auto arrived = [&]() {
+          ok = mbar_wait(&full[slot], phase, err, 3);
+          if (ok) tc_fence_after();
+          return ok;
+        };
+        auto advance = [&]() {
+          if (++slot == ring) {
+            slot = 0;
+            phase ^= 1u;
+          }
+        };
+        if constexpr (NPIECE == 3) {  // piece pairs of order >= 2^-16, and (2, 1)
+          for (int kc = 0; kc < nfull && ok; ++kc) {
+            if (fresh) ok = mbar_wait(&bfull[kc], (uint32_t)(nb - 1) & 1u, err, 3);
+            for (int q = 1; q < 3 && ok; ++q) {
+              if (!arrived()) break;
+              steps(slot, kc, 0, kIdesc256, kc == 0 && q == 1);
+              mma_commit(&empty[slot]);
+              advance();
             }
+          }
+          int held = slot;  // of the first piece 0
+          for (int kc = 0; kc < nfull && ok; ++kc) {
+            if (!arrived()) break;
+            steps(slot, kc, 0, kIdesc256, false);
+            advance();
+          }
+          if (!ok) break;
+          mma_commit(wide);
+          ok = mbar_wait(wide, wphase, err, 8);
+          if (!ok) break;
+          wphase ^= 1u;
+          tc_fence_after();
+          for (int kc = 0; kc < nfull; ++kc) {
+            steps(held, kc, 2, kIdesc, false);
+            mma_commit(&empty[held]);
             if (last) mma_commit(&bempty[kc]);
-            continue;
+            if (++held == ring) held = 0;
           }
-          // piece pairs of order >= 2^-16
-#pragma unroll
-          for (int i = 0; i < NPIECE; ++i) {
-            const int qa = a_piece(NPIECE, i);
-            ok = mbar_wait(&full[slot], phase, err, 3);
-            if (!ok) break;
-            tc_fence_after();
+          if (packed) {  // piece q is K step q of the one tile
+            if (fresh) ok = mbar_wait(&bfull[nfull], (uint32_t)(nb - 1) & 1u, err, 3);
+            if (!ok || !arrived()) break;
             const uint64_t da = make_desc(smem_u32(sA) + (uint32_t)slot * kTileBytes);
-            auto steps = [&](int qb, uint32_t idesc) {
-              const uint64_t db = make_desc(b0 + qb * kTileBytes);
+            const uint64_t db = make_desc(smem_u32(sB) + (uint32_t)(nfull * NPIECE) * kTileBytes);
 #pragma unroll
-              for (int kk = 0; kk < kChunkK / 16; ++kk)
-                if (kk < ksteps)
-                  mma_bf16(d_tmem, da + (uint64_t)(kk * 2), db + (uint64_t)(kk * 2),
-                           (kc > 0 || i > 0 || kk > 0) ? 1u : 0u, idesc);
-            };
-            if constexpr (NPIECE == 3) {
-              if (qa == 0) steps(2, kIdesc);
-              steps(0, qa == 2 ? kIdesc : kIdesc256);
-            } else {
-              steps(0, kIdesc);
-            }
+            for (int qa = 2; qa >= 0; --qa)
+#pragma unroll
+              for (int qb = 2 - qa; qb >= 0; --qb)
+                mma_bf16(d_tmem, da + (uint64_t)(qa * 2), db + (uint64_t)(qb * 2), 1u);
             mma_commit(&empty[slot]);
-            if (++slot == ring) {
-              slot = 0;
-              phase ^= 1u;
-            }
+            if (last) mma_commit(&bempty[nfull]);
+            advance();
           }
-          if (ok && last) mma_commit(&bempty[kc]);
+        } else {
+          for (int kc = 0; kc < nkc && ok; ++kc) {
+            if (fresh) ok = mbar_wait(&bfull[kc], (uint32_t)(nb - 1) & 1u, err, 3);
+            if (!ok || !arrived()) break;
+            steps(slot, kc, 0, kIdesc, kc == 0);
+            mma_commit(&empty[slot]);
+            advance();
+            if (last) mma_commit(&bempty[kc]);
+          }
         }
         if (!ok) break;
         mma_commit(&tfull[acc]);
@@ -661,7 +689,7 @@ size_t smem_bytes() {
   return 1024 + (size_t)NSTAGE * 2 * NPIECE * kTileBytes + 8 * (2 * NSTAGE + 5) + 16;
 }
 
-constexpr size_t kResidentSmem = 1024 + (size_t)kSlots * kTileBytes + 8 * (2 * (kSlots + kResidentMax) + 5) + 16;
+constexpr size_t kResidentSmem = 1024 + (size_t)kSlots * kTileBytes + 8 * (2 * (kSlots + kResidentMax) + 6) + 16;
 
 template <int NPIECE>
 cudaError_t launch(const SuperposeArgs& a, int64_t grid, int32_t* err, cudaStream_t st) {

@@ -1,4 +1,6 @@
-"""Superpositions whose tensor-core products share an accumulator give the same bits on every call: the FP64 digit form. Against the FP64 product of basis and
+"""Superpositions whose tensor-core products share an accumulator give the same bits on every call:
+the FP64 digit form, and the resident column tile with its two widths of product (2 and 3 K chunks,
+a packed last chunk or not, one column tile and several). Against the FP64 product of basis and
 currents: 1e-6 for MTS_MIXED and 1e-12 for MTS_FP64."""
 import numpy as np
 import pytest
@@ -14,6 +16,12 @@ from paper_2503_18479_gb300.simulator import Simulator  # noqa: E402
 @pytest.mark.parametrize("nx,ny,P,n_cfg,precision", [
     (8, 8, 9000, 320, "fp64"),
     (13, 11, 4000, 100, "fp64"),
+    (13, 5, 12000, 500, "mixed"),   # 65 ports: one full chunk, one packed
+    (13, 10, 12000, 500, "mixed"),  # 130: two full, one packed
+    (15, 10, 12000, 60, "mixed"),   # 150: three full
+    (12, 16, 9000, 500, "mixed"),   # 192: three full
+    (13, 8, 12000, 500, "mixed"),   # 104: two full
+    (20, 10, 12000, 500, "bf16"),
 ])
 def test_repeated_calls(nx, ny, P, n_cfg, precision):
     rng = np.random.default_rng(1)
