@@ -23,9 +23,9 @@ def _basis(loops, pts, precision):
 def test_point_order(precision):
     rng = np.random.default_rng(0)
     loops = W.square_array(1, 1, seg_per_side=4) + [W.circular_loop(.034, 33)]
-    # all around the distance where the form changes (twice that of the furthest vertex)
+    # all around the distance where the form changes (three times that of the furthest vertex)
     pts = rng.standard_normal((1000, 3))
-    pts *= (rng.uniform(.05, .1, 1000) / np.linalg.norm(pts, axis=1))[:, None]
+    pts *= (rng.uniform(.07, .15, 1000) / np.linalg.norm(pts, axis=1))[:, None]
     H = _basis(loops, pts, precision)
     order = rng.permutation(len(pts))
     assert np.array_equal(_basis(loops, pts[order], precision), H[order])
