@@ -15,12 +15,6 @@ struct cd {
   double x, y;
 };
 __device__ inline cd cmul(cd a, cd b) { return {a.x * b.x - a.y * b.y, a.x * b.y + a.y * b.x}; }
-__device__ inline cd csub(cd a, cd b) { return {a.x - b.x, a.y - b.y}; }
-__device__ inline cd cadd(cd a, cd b) { return {a.x + b.x, a.y + b.y}; }
-__device__ inline cd cdiv(cd a, cd b) {
-  double d = b.x * b.x + b.y * b.y;
-  return {(a.x * b.x + a.y * b.y) / d, (a.y * b.x - a.x * b.y) / d};
-}
 __device__ inline double cabs2(cd a) { return a.x * a.x + a.y * a.y; }
 
 // Objective term of one loss point and its cotangent G = de/dRe b + j de/dIm b.
@@ -193,21 +187,6 @@ __device__ inline SysInfo sys_info(const SolveArgs& a, int64_t sys) {
   si.N = a.port_off[si.s + 1] - si.k0;
   si.w = a.omega[si.g];
   return si;
-}
-
-
-// error-free product and sum on the FP32 pipe: (sh, sl) += (ah + al) * (bh + bl), dropping
-// al * bl (2^-48 relative)
-__device__ inline void df_mac(float& sh, float& sl, float ah, float al, float bh, float bl) {
-  float p = ah * bh;
-  float e = fmaf(ah, bh, -p);
-  e = fmaf(ah, bl, e);
-  e = fmaf(al, bh, e);
-  float t = sh + p;
-  float z = t - sh;
-  float err = (sh - (t - z)) + (p - z);
-  sh = t;
-  sl += err + e;
 }
 
 }  // namespace mts
