@@ -57,11 +57,14 @@ typedef enum {
 
 typedef enum {
   /* FP64 everywhere: basis, FP64 LU with partial pivoting, FP64 superposition;
-     B_out is complex128. Target error against the FP64 oracle <= 1e-10. */
+     B_out is complex128. Target error against the FP64 oracle <= 1e-10. Every value of B is
+     as accurate as a plain FP64 sum of its N products, relative to sum |H_k I_k|, also where
+     the sum is formed on the tensor cores (exact products of 8-bit digits). */
   MTS_FP64 = 0,
   /* FP32 basis with FP64 near-field terms; FP32 complex LU with partial pivoting and
-     iterative refinement on residuals taken in FP64-equivalent precision; superposition
-     on the tensor cores with three-way bf16 operand splitting and FP32 accumulation;
+     iterative refinement on residuals in pairs of FP32 numbers (about 2^-46, the FP32
+     exponent range; currents and losses are accumulated so too); superposition on
+     the tensor cores with three-way bf16 operand splitting and FP32 accumulation;
      B_out is complex64. Target error <= 1e-6. */
   MTS_MIXED = 1,
   /* As MTS_MIXED but the superposition uses single bf16 operands (one tensor-core pass);

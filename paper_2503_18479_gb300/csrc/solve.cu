@@ -28,9 +28,9 @@ namespace mts {
 //
 // The bound is the FP64 pipe (a warp's instruction holds it for 16 cycles): about 21,000 of its
 // instructions a 64-port system, 16,000 of them the LU's updates. Everything else on a pivot step
-// is kept off that pipe or shared: the pivot search runs on the high words of |a|^2 (20 bits of
-// mantissa decide, which row of nearly equal ones is taken does not matter) with the row in the
-// low bits, by one redux; a step divides once, by |pivot|^2, and keeps the inverse pivot on the
+// is kept off that pipe or shared: the pivot search runs on the high words of |a|^2 with the row in
+// their low bits, by one redux (13 bits of mantissa decide: of rows within 2^-13 the first is
+// taken, so that multipliers stay below 1 + 2^-14); a step divides once, by |pivot|^2, and keeps the inverse pivot on the
 // diagonal for the solves; one barrier a step, because a chosen row is never written again and
 // the search words alternate by step parity. 1024 systems of 64 ports with objective and
 // adjoint: 3030 us with two divisions a row and step, FP64 compares and three barriers.

@@ -4,8 +4,10 @@
 //   plan_kernel          per-call tables: bases of the tensor-core operand of I, the
 //                        prefix of GEMM work units and the bases of the LU factor scratch
 //                        per structure
-//   superpose_simt_kernel  SIMT: MTS_FP64, and structures with at most 16 systems
-//   The tensor-core kernel for MTS_MIXED / MTS_BF16 lives in superpose_tc.cu.
+//   superpose_simt_kernel  SIMT: structures with at most 16 systems; MTS_FP64 with several
+//                        structures, or where its tensor-core form is the slower one
+//   The tensor-core kernels live in superpose_tc.cu (MTS_MIXED, MTS_BF16) and
+//   superpose_fp64_tc.cu (MTS_FP64, one structure).
 #include <cuda_runtime.h>
 
 #include "common.cuh"
@@ -124,9 +126,10 @@ cudaError_t launch_plan(const mts_problem* pb, int64_t n_cfg, int npieces, int64
 // otherwise each thread reads its own row of H straight from global memory.
 // The currents of the unit's systems are staged per K chunk in shared memory (k-major: the
 // systems of one k are contiguous, read as broadcasts). Used for MTS_FP64 (T = double, FP64
-// basis) and, in the other precisions, for structures with at most 16 systems (T = float,
-// FP32 basis, FP32 accumulation), where tensor-core column tiles would be mostly padding and
-// the work is a read of H.
+// basis) with several structures, and with one where superpose_fp64_tc_units prefers it (few ports,
+// small batches), and, in the other precisions, for structures with at most 16 systems (T =
+// float, FP32 basis, FP32 accumulation), where tensor-core column tiles would be mostly padding
+// and the work is a read of H.
 template <typename T>
 struct SimtCfg;
 template <>
