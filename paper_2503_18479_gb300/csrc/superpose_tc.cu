@@ -413,7 +413,7 @@ constexpr int kResidentMax = 9;  // of them at most for the column tile
 // An MMA of M = 128 takes much the same time for N = 128 and N = 256, so the products of an A
 // piece with the first two B pieces go out as one MMA of N = 256: the pieces' tiles follow each
 // other in shared memory as the rows of one operand, and the second one's products have an
-// accumulator of their own, which the epilogue adds (65,600 points below: 783 -> 733 us).
+// accumulator of their own, which the epilogue adds (65,600 points below: 783 -> 726 us).
 //
 // MMAs are only sure to run in order on one accumulator in one shape. So a unit's products of
 // N = 256 (every A piece with B pieces 0 and 1) go out first, and when they are done those of
@@ -421,11 +421,11 @@ constexpr int kResidentMax = 9;  // of them at most for the column tile
 // and 2 of every full chunk, then their pieces 0, whose slots are held until both shapes have
 // read them (at most three of five slots or more), then the last chunk. The products of N = 128 go
 // to the second accumulator, which is small: added to the first one, behind the largest products,
-// they put B of 80 ports 2.6e-7 off instead of 1.7e-7. The wait itself costs
-// nothing (the bound is the latency of the point tiles, 16 KB each, over the ring's slots), the
-// held slots do: 651 us in the order of arrival against 733 us, 282 against 323 us for half the
-// columns at K = 104. A tile of zeros beside the third pieces, which makes their products N = 256 too, takes a
-// slot for good: 734 and 305 us, 534 against 513 us at K = 192.
+// they put B of 80 ports 2.6e-7 off instead of 1.7e-7.
+// The wait itself costs nothing (the bound is the latency of the point tiles, 16 KB each, over the
+// ring's slots), the held slots do: 651 us in the order of arrival against 726 us, 282 against
+// 321 us for half the columns at K = 104. A tile of zeros beside the third pieces, which makes their
+// products N = 256 too, takes a slot for good: 734 and 305 us, 534 against 511 us at K = 192.
 constexpr uint32_t kIdesc256 = (kIdesc & ~(0x3fu << 17)) | ((256u >> 3) << 17);
 
 // 16 KB tiles that one side of a unit takes
